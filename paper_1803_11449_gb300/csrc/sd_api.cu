@@ -248,6 +248,7 @@ struct sd_handle {
     PlaneArgs pa{};                    // counters and plane copy (bins, tile, unit set per round)
     bool planes_dirty = false;
     bool grid_clean = false;           // the DHLA is all zero (reset, then plane updates only)
+    bool grid_stale = false;           // the DHLA is empty but its words hold an earlier close's bits
     uint64_t plane_prev_pairs = 0;     // pairs of the round whose counts are in prev (0: none)
     int plane_layout_view = -2;        // its directions (-1 both, else one)
 
@@ -738,11 +739,22 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
     return SD_OK;
 }
 
+// The DHLA's words as they should be (stream-ordered): zero where a close
+// left them stale.
+static int freshen_grid(sd_handle *h) {
+    if (!h->grid_stale) return SD_OK;
+    SD_CK(h, cudaMemsetAsync(h->grid, 0, (uint64_t)h->G.dirs * h->G.dir_words * 4, h->stream));
+    h->grid_stale = false;
+    h->grid_clean = true;
+    return SD_OK;
+}
+
 // grid |= planes^T and planes = 0 (stream-ordered), when updates of the
 // plane-binned mode are pending.
 static int fold_planes(sd_handle *h) {
-    if (!h->planes_dirty) return SD_OK;
-    const FoldJob job{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot, nullptr, nullptr};
+    const int rc = freshen_grid(h);
+    if (rc != SD_OK || !h->planes_dirty) return rc;
+    const FoldJob job{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot, nullptr, nullptr, nullptr};
     SD_CK(h, launch_plane_fold(job, nullptr, 1, h->G, h->pa.ps, h->num_sms, h->stream));
     launched(1);
     h->planes_dirty = false;
@@ -771,6 +783,8 @@ static int update_device(sd_handle *h, const uint32_t *pairs, uint64_t n, int di
         if (rc != SD_OK) return rc;
         return plane_rounds(h, pairs, n, dir, h->plane_bins, h->plane_bins_words, round, h->stream, h);
     }
+    const int frc = freshen_grid(h);
+    if (frc != SD_OK) return frc;
     h->grid_clean = false;  // the other modes set bits in the DHLA itself
     if (h->T.mode == 5) {
         bool ok = false;
@@ -1103,6 +1117,8 @@ int sd_update_many(sd_handle *const *hs, const uint32_t *const *pairs, const uin
     // the members' earlier work comes first, on the driver's stream
     for (uint32_t q : batch) {
         sd_handle *h = hs[q];
+        const int frc = freshen_grid(h);
+        if (frc != SD_OK) return frc;
         if (h == d || h->stream == d->stream) continue;
         SD_CK(h, cudaEventRecord(h->ev_batch, h->stream));
         SD_CK(d, cudaStreamWaitEvent(d->stream, h->ev_batch, 0));
@@ -1222,21 +1238,31 @@ static int close_phase_a(sd_handle *h, sd_report *out) {
     std::memset(&h->cs, 0, sizeof h->cs);
     h->report.clear();
     h->last_ncand[0] = h->last_ncand[1] = 0;
-    if (h->planes_dirty && fold_stats_fit(h->G)) {
-        // the fold writes the row statistics as it goes
-        const FoldJob job{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot, h->st_d, h->hotmap};
-        SD_CK(h, launch_plane_fold(job, nullptr, 1, h->G, h->pa.ps, h->num_sms, h->stream));
+    if (h->planes_dirty && fold_stats_fit(h->G) && (h->grid_clean || h->grid_stale)) {
+        // the whole DHLA is the plane copy: counted as it is
+        const FoldJob job{h->grid, h->planes, 1u, h->zhot, h->st_d, h->hotmap, h->he};
+        SD_CK(h, launch_plane_scan(job, nullptr, 1, h->G, h->pa.ps, h->stream));
         launched(1);
         h->planes_dirty = false;
         h->grid_clean = false;
+        h->grid_stale = true;
     } else {
-        const int frc = fold_planes(h);
-        if (frc != SD_OK) return frc;
-        SD_CK(h, launch_row_stats(h->grid, h->G, h->zhot, h->hotmap, h->st_d, h->num_sms, h->stream));
+        if (h->planes_dirty && fold_stats_fit(h->G)) {
+            // the fold writes the row statistics as it goes
+            const FoldJob job{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot, h->st_d, h->hotmap, nullptr};
+            SD_CK(h, launch_plane_fold(job, nullptr, 1, h->G, h->pa.ps, h->num_sms, h->stream));
+            launched(1);
+            h->planes_dirty = false;
+            h->grid_clean = false;
+        } else {
+            const int frc = fold_planes(h);
+            if (frc != SD_OK) return frc;
+            SD_CK(h, launch_row_stats(h->grid, h->G, h->zhot, h->hotmap, h->st_d, h->num_sms, h->stream));
+            launched(1);
+        }
+        SD_CK(h, launch_compact(h->hotmap, h->G, h->he, 2, h->stream));
         launched(1);
     }
-    SD_CK(h, launch_compact(h->hotmap, h->G, h->he, 2, h->stream));
-    launched(1);
     SD_CK(h, cudaMemcpyAsync(h->st_h, h->st_d, sizeof(StatBlock), cudaMemcpyDeviceToHost, h->stream));
     return SD_OK;
 }
@@ -1433,7 +1459,9 @@ static int close_phase_d(sd_handle *h, sd_report *out, bool reset = true) {
     h->have_close = true;
     // clear the DHLA and the counters for the next window (stream-ordered;
     // a batched close clears all its handles in one launch instead)
-    if (reset) {
+    if (reset && h->grid_stale) {
+        SD_CK(h, cudaMemsetAsync(h->st_d, 0, sizeof(StatBlock), h->stream));
+    } else if (reset) {
         SD_CK(h, launch_reset(h->grid, (uint64_t)G.dirs * G.dir_words, h->st_d, h->num_sms, h->stream));
         launched(1);
         h->grid_clean = !h->planes_dirty;
@@ -1566,21 +1594,46 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
     // on the driver's stream, which is ordered after every member's work)
     // (with the row statistics where the shape allows: those members skip
     // k_row_stats_many)
-    uint32_t nfold = 0;
+    // (members whose whole DHLA is their plane copy: counted as it is; the
+    // others folded with the row statistics, where the shape allows)
     const bool fold_stats = fold_stats_fit(G);
     std::vector<char> folded(count, 0);
+    uint32_t nscan = 0, nfold = 0;
+    bool any_fresh = false;
     for (uint32_t i = 0; i < count; i++) {
         sd_handle *h = hs[i];
-        if (!h->planes_dirty) continue;
-        d->fj_h[nfold++] = FoldJob{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot,
-                                   fold_stats ? h->st_d : nullptr, fold_stats ? h->hotmap : nullptr};
-        folded[i] = fold_stats;
-        h->planes_dirty = false;
-        h->grid_clean = false;
+        if (h->planes_dirty && fold_stats && (h->grid_clean || h->grid_stale)) folded[i] = 2, nscan++;
+        else any_fresh = true;
+    }
+    for (uint32_t i = 0, at = 0; i < count; i++) {
+        sd_handle *h = hs[i];
+        if (folded[i] == 2) {
+            d->fj_h[at++] = FoldJob{h->grid, h->planes, 1u, h->zhot, h->st_d, h->hotmap, h->he};
+            h->planes_dirty = false;
+            h->grid_clean = false;
+            h->grid_stale = true;
+        } else {
+            if (h->grid_stale)
+                SD_CK(d, cudaMemsetAsync(h->grid, 0, (uint64_t)G.dirs * G.dir_words * 4, s));
+            h->grid_clean = h->grid_clean || h->grid_stale;
+            h->grid_stale = false;
+            if (!h->planes_dirty) continue;
+            d->fj_h[nscan + nfold++] = FoldJob{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot,
+                                               fold_stats ? h->st_d : nullptr, fold_stats ? h->hotmap : nullptr,
+                                               nullptr};
+            folded[i] = fold_stats;
+            h->planes_dirty = false;
+            h->grid_clean = false;
+        }
+    }
+    if (nscan + nfold)
+        SD_CK(d, cudaMemcpyAsync(d->fj_d, d->fj_h, (nscan + nfold) * sizeof(FoldJob), cudaMemcpyHostToDevice, s));
+    if (nscan) {
+        SD_CK(d, launch_plane_scan(d->fj_h[0], d->fj_d, nscan, G, plane_words(G), s));
+        launched(1);
     }
     if (nfold) {
-        SD_CK(d, cudaMemcpyAsync(d->fj_d, d->fj_h, nfold * sizeof(FoldJob), cudaMemcpyHostToDevice, s));
-        SD_CK(d, launch_plane_fold(d->fj_h[0], d->fj_d, nfold, G, plane_words(G), d->num_sms, s));
+        SD_CK(d, launch_plane_fold(d->fj_h[nscan], d->fj_d + nscan, nfold, G, plane_words(G), d->num_sms, s));
         launched(1);
     }
     for (uint32_t i = 0; i < count; i++) {
@@ -1601,9 +1654,12 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         rcs[i] = SD_OK;
     }
     SD_CK(d, cudaMemcpyAsync(d->cj_d, d->cj_h, count * sizeof(CloseJob), cudaMemcpyHostToDevice, s));
-    SD_CK(d, launch_stats_many(d->cj_d, count, G, d->num_sms, s));
+    if (any_fresh) {
+        SD_CK(d, launch_stats_many(d->cj_d, count, G, d->num_sms, s));
+        launched(2);
+    }
     SD_CK(d, launch_gather_many(d->cj_d, count, d->cb_st_d, d->cb_hits_d, s));
-    launched(3);
+    launched(1);
     SD_CK(d, cudaMemcpyAsync(d->cb_st_h, d->cb_st_d, count * sizeof(StatBlock), cudaMemcpyDeviceToHost, s));
     SD_CK(d, cudaStreamSynchronize(s));
     tr.mark(0);
@@ -1657,7 +1713,7 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         if (rcs[i] == SD_OK) rcs[i] = close_phase_d(hs[i], &outs[i], false);
     SD_CK(d, launch_reset_many(d->cj_d, count, G, d->num_sms, s));
     launched(1);
-    for (uint32_t i = 0; i < count; i++) hs[i]->grid_clean = !hs[i]->planes_dirty;
+    for (uint32_t i = 0; i < count; i++) hs[i]->grid_clean = !hs[i]->grid_stale && !hs[i]->planes_dirty;
     tr.mark(3);
     // each member's later work waits for the batch
     SD_CK(d, cudaEventRecord(d->ev_batch, s));
@@ -1823,17 +1879,27 @@ int sd_merge(sd_handle *dst, sd_handle *src) {
         a.device != b.device)
         return dst->fail(SD_ERR_ARG, "sd_merge: handles differ in shape, seed or device");
     DeviceGuard dg(a.device);
-    int frc = fold_planes(src);
-    if (frc == SD_OK) frc = fold_planes(dst);
-    if (frc != SD_OK) return frc;
-    dst->grid_clean = false;
+    // two DHLAs that are plane copies and nothing else are merged as such:
+    // no fold, and dst's close still counts its plane copy
+    const bool as_planes = src->planes_dirty && (src->grid_clean || src->grid_stale) && dst->planes &&
+                           (dst->grid_clean || dst->grid_stale);
+    if (!as_planes) {
+        int frc = fold_planes(src);
+        if (frc == SD_OK) frc = fold_planes(dst);
+        if (frc != SD_OK) return frc;
+        dst->grid_clean = false;
+    }
     cudaEvent_t ev;
     SD_CK(dst, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     cudaError_t e = cudaEventRecord(ev, src->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(dst->stream, ev, 0);
     if (e == cudaSuccess) {
-        e = launch_merge(dst->grid, src->grid, (uint64_t)a.dirs * dst->G.dir_words, dst->num_sms, dst->stream);
+        if (as_planes)
+            e = launch_merge(dst->planes, src->planes, (uint64_t)dst->pa.nbins * dst->pa.ps, dst->num_sms, dst->stream);
+        else
+            e = launch_merge(dst->grid, src->grid, (uint64_t)a.dirs * dst->G.dir_words, dst->num_sms, dst->stream);
         if (e == cudaSuccess) launched(1);
+        if (e == cudaSuccess && as_planes) dst->planes_dirty = true;
     }
     if (e == cudaSuccess) e = cudaEventRecord(ev, dst->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(src->stream, ev, 0);  // src may not change until merged

@@ -837,6 +837,7 @@ __global__ void __launch_bounds__(256) k_row_stats_many(const CloseJob *__restri
 
 __global__ void __launch_bounds__(1024) k_compact_many(const CloseJob *__restrict__ J) {
     const CloseJob &j = J[blockIdx.y];
+    if (j.stats_done == 2) return;  // listed by k_plane_scan
     compact_body(j.A.hotmap, j.G, const_cast<uint32_t *>(j.A.he), 2, blockIdx.x);
 }
 
@@ -965,7 +966,9 @@ k_gather_many(const CloseJob *__restrict__ J, StatBlock *__restrict__ st_out, un
 
 __global__ void k_reset_many(const CloseJob *__restrict__ J, uint64_t n4) {
     const CloseJob &j = J[blockIdx.y];
-    reset_body(reinterpret_cast<uint4 *>(const_cast<uint32_t *>(j.A.grid)), n4, j.A.stats, blockIdx.x, gridDim.x);
+    // a DHLA that k_plane_scan wrote holds hot estimators' bits only: stale, not to be cleared
+    reset_body(reinterpret_cast<uint4 *>(const_cast<uint32_t *>(j.A.grid)), j.stats_done == 2 ? 0 : n4, j.A.stats,
+               blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------- launchers

@@ -116,6 +116,7 @@ struct StatBlock {
     unsigned int big_sort[2];  // 1: hits did not fit the one-block sort
     unsigned int pad[2];
     unsigned long long jcount[2][kMaxRows];  // staged join: entries stage i produced
+    unsigned int rows_done[2][2];  // k_plane_scan: tiles of rows 0 and 1 counted
 };
 
 struct RestoreArgs {
@@ -144,7 +145,8 @@ struct CloseJob {
     Geometry G;
     RestoreArgs A;
     int zhot;
-    int stats_done;  // the fold already wrote the row statistics
+    int stats_done;  // 0: to be computed from the DHLA; 1: the fold wrote the row statistics;
+                     // 2: k_plane_scan wrote them, HE(0) and HE(1) (the DHLA need not be cleared)
 };
 
 // The staged join of sd_join.cu (the paper's Algorithms 3 and 4).
@@ -234,7 +236,7 @@ void geometry_of(const sd_params *p, Geometry *out);
 // used for grid sizing): row stats + HE(0), HE(1) of every job; restore,
 // estimate and small sorts; a gather of every job's StatBlock and first
 // kSortSmall hits per direction into st_out[count] / hits_out[count][2]
-// [kSortSmall]; the reset of every job's DHLA and counters.
+// [kSortSmall]; the reset of every job's counters and (stats_done < 2) DHLA.
 cudaError_t launch_stats_many(const CloseJob *J, uint32_t count, const Geometry &G, int num_sms, cudaStream_t s);
 void prepare_restore(const Geometry &G, RestoreArgs &A, int num_sms, uint32_t tiles_per_block);
 // (restore and estimate spread all jobs' tiles / candidates over the whole
@@ -288,6 +290,7 @@ struct FoldJob {
     int zhot;
     StatBlock *st;       // nullptr: no statistics
     uint32_t *hotmap;    // [dirs][r][2^k/32]
+    uint32_t *he;        // [dirs][2][2^k] (k_plane_scan)
 };
 // Whether a fold can compute the row statistics: tiles then hold every bit
 // of their estimators (g/32 words of 8, 16 or 32).
@@ -295,6 +298,12 @@ inline bool fold_stats_fit(const Geometry &G) { return G.wpc >= 8 && G.wpc <= 32
 // `one`'s fold, or (jobs != nullptr) the folds of njobs device-resident jobs
 cudaError_t launch_plane_fold(const FoldJob &one, const FoldJob *jobs, uint32_t njobs, const Geometry &G, uint32_t ps,
                               int num_sms, cudaStream_t s);
+// A close's counting pass over the plane copy of a handle whose DHLA is empty
+// (`one`, or njobs device-resident jobs): row statistics, hot bitmaps,
+// HE(0) and HE(1), the hot estimators' bits in the DHLA, planes = 0; where
+// fold_stats_fit.
+cudaError_t launch_plane_scan(const FoldJob &one, const FoldJob *jobs, uint32_t njobs, const Geometry &G, uint32_t ps,
+                              cudaStream_t s);
 cudaError_t launch_binned_chunk(const uint32_t *pairs, uint64_t n, uint32_t *grid, const Geometry &G,
                                 const BinArgs &B, int num_sms, cudaStream_t s);
 cudaError_t launch_binned_links(const LinkDesc *links_dev, uint32_t nlinks, uint64_t ntiles_all,

@@ -254,4 +254,230 @@ cudaError_t launch_plane_fold(const FoldJob &one, const FoldJob *jobs, uint32_t 
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------- fold at a close
+// A window close reads the DHLA twice: for every estimator's z_0, and for
+// the bits of the hot ones (each candidate's r estimators are hot).  So when
+// the DHLA holds nothing but the plane copy, the close does not fold it: it
+// counts every estimator's bits in the plane copy as it is, clears the copy,
+// and writes only the hot estimators' bits to the DHLA.  The other words of
+// the DHLA keep what an earlier close left there and the handle is marked
+// stale: the next close writes all that it reads, and any other reader
+// clears the DHLA first.  HE(0) and HE(1) are listed by the block that
+// counts the last estimators of their row.
+//
+// Counting: a thread holds one word (32 estimators) of 32 planes and adds
+// them bit-sliced (57 full adders of two three-input operations each give
+// six words: bit i of word b is bit b of estimator i's count); the g/32
+// partial counts of a word are added the same way through shared memory, and
+// the hot test z_0 <= zhot, i.e. count >= g - zhot, is a bit-sliced
+// comparison.  No transpose, except of the 32 x 32 blocks whose word has a
+// hot estimator.  Bound by the plane copy's read and clear: the core
+// sketch's 32 MiB take 16 us with few hot estimators and 22 us with 4,200 a
+// row (the fold with statistics, the lists and the DHLA's clear took 28 to
+// 33, 4 and 6.5 us); 64 of them 0.96 ms (1.4 and 0.3 ms), 4.5 TB/s.
+constexpr uint32_t kScanThreads = 256;
+constexpr uint32_t kCountBits = 12;  // counts up to 1024
+
+// s = a + b of N-bit sliced numbers, N + 1 bits
+template <int N>
+__device__ __forceinline__ void add_sliced(const uint32_t (&a)[N], const uint32_t (&b)[N], uint32_t (&s)[N + 1]) {
+    uint32_t carry = 0;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        s[i] = a[i] ^ b[i] ^ carry;
+        carry = (a[i] & b[i]) | (carry & (a[i] ^ b[i]));
+    }
+    s[N] = carry;
+}
+
+// bit-sliced sum of x[at .. at + 2^LOG)
+template <int LOG>
+__device__ __forceinline__ void count_sliced(const uint32_t (&x)[32], int at, uint32_t (&s)[LOG + 1]) {
+    if constexpr (LOG == 0) {
+        s[0] = x[at];
+    } else {
+        uint32_t a[LOG], b[LOG];
+        count_sliced<LOG - 1>(x, at, a);
+        count_sliced<LOG - 1>(x, at + (1 << (LOG - 1)), b);
+        add_sliced<LOG>(a, b, s);
+    }
+}
+
+// HE(row) of direction d in ascending order from its hot bitmap (one block;
+// the bitmap words were written by other blocks).
+__device__ __forceinline__ void list_hot(const uint32_t *bm, uint32_t nw, uint32_t *out) {
+    __shared__ uint32_t s_tot[kScanThreads / 32];
+    const uint32_t per = (nw + blockDim.x - 1) / blockDim.x;
+    const uint32_t w0 = min(threadIdx.x * per, nw), w1 = min(w0 + per, nw);
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    uint32_t cnt = 0;
+    for (uint32_t w = w0; w < w1; w++) cnt += __popc(__ldcg(bm + w));
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if ((int)lane >= o) incl += v;
+    }
+    if (lane == 31) s_tot[wid] = incl;
+    __syncthreads();
+    uint32_t pos = incl - cnt;
+    for (uint32_t q = 0; q < wid; q++) pos += s_tot[q];
+    for (uint32_t w = w0; w < w1; w++) {
+        uint32_t b = __ldcg(bm + w);
+        while (b) {
+            out[pos++] = (w << 5) | (uint32_t)(__ffs(b) - 1);
+            b &= b - 1u;
+        }
+    }
+    __syncthreads();
+}
+
+// p, with its value hidden from the compiler: a later pass over the same 32
+// addresses then forms them again instead of keeping them in 64 registers.
+__device__ __forceinline__ uint32_t *opaque(uint32_t *p) {
+    asm volatile("" : "+l"(p));
+    return p;
+}
+
+// TC = g/32 plane groups; a block takes W = 256 / TC words of one row.
+template <int TC>
+__global__ void __launch_bounds__(kScanThreads, 4)
+k_plane_scan(FoldJob one, const FoldJob *__restrict__ jobs, Geometry G, uint32_t ps) {
+    constexpr uint32_t W = kScanThreads / TC;
+    constexpr int LOG = TC == 8 ? 3 : TC == 16 ? 4 : 5;  // log2 TC
+    constexpr int LW = LOG - 3;                          // of them within a warp
+    constexpr int S = 6 + LOG;                           // bits of a full count
+    __shared__ uint32_t s_part[7][S][W];
+    __shared__ uint32_t s_hot[W];
+    __shared__ bool s_list;
+    const uint32_t rw = (1u << G.k) >> 5;
+    const uint32_t wgroups = (rw + W - 1) / W;
+    uint32_t tile = blockIdx.x;
+    const uint32_t wg = tile % wgroups;
+    tile /= wgroups;
+    const uint32_t i = tile % G.r;
+    tile /= G.r;
+    const uint32_t d = tile % G.dirs;
+    const FoldJob job = jobs ? jobs[tile / G.dirs] : one;
+    const uint32_t tt = threadIdx.x / W, w = threadIdx.x % W, word = wg * W + w;
+    const bool live = word < rw;
+    uint32_t *src = job.planes + ((uint64_t)d * G.g + 32u * tt) * ps + (uint64_t)i * rw + word;
+    uint32_t acc[S];  // this thread's count, then sums of TC of them
+    uint32_t any = 0;  // planes with a bit in this word
+    {
+        uint32_t x[32], mine[6];
+        const uint32_t *p = src;
+#pragma unroll
+        for (uint32_t j = 0; j < 32; j++, p += ps) x[j] = live ? __ldcg(p) : 0u;
+#pragma unroll
+        for (uint32_t j = 0; j < 32; j++) any |= (x[j] ? 1u : 0u) << j;
+        count_sliced<5>(x, 0, mine);
+#pragma unroll
+        for (int b = 0; b < S; b++) acc[b] = b < 6 ? mine[b] : 0u;
+    }
+    // the plane groups within a warp, then the eight warps, pairwise
+#pragma unroll
+    for (int l = 0; l < LW; l++) {
+        uint32_t v[S - 1];
+#pragma unroll
+        for (int b = 0; b < 6 + l; b++) v[b] = __shfl_xor_sync(0xFFFFFFFFu, acc[b], W << l);
+        uint32_t carry = 0;
+#pragma unroll
+        for (int b = 0; b < 6 + l; b++) {
+            const uint32_t a = acc[b];
+            acc[b] = a ^ v[b] ^ carry;
+            carry = (a & v[b]) | (carry & (a ^ v[b]));
+        }
+        acc[6 + l] = carry;
+    }
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int l = 0; l < 3; l++) {
+        const uint32_t half = 4u >> l, at = 8u - 2u * half;  // slots at, at + 1, ... of this level
+        if (wid >= half && wid < 2 * half && lane < W) {
+#pragma unroll
+            for (int b = 0; b < 6 + LW + l; b++) s_part[at + wid - half][b][lane] = acc[b];
+        }
+        __syncthreads();
+        if (wid < half && lane < W) {
+            uint32_t carry = 0;
+#pragma unroll
+            for (int b = 0; b < 6 + LW + l; b++) {
+                const uint32_t v = s_part[at + wid][b][lane], a = acc[b];
+                acc[b] = a ^ v ^ carry;
+                carry = (a & v) | (carry & (a ^ v));
+            }
+            acc[6 + LW + l] = carry;
+        }
+    }
+    if (threadIdx.x < W) {  // lanes of the first warp
+        const uint32_t T = (uint32_t)max((int)G.g - job.zhot, 0);
+        uint32_t gt = 0, eq = ~0u, ones = 0;
+#pragma unroll
+        for (int b = kCountBits - 1; b >= 0; b--) {
+            const uint32_t v = b < S ? acc[b < S ? b : 0] : 0u;
+            const uint32_t t = (T >> b & 1u) ? ~0u : 0u;
+            gt |= eq & v & ~t;
+            eq &= ~(v ^ t);
+            ones += (uint32_t)__popc(v) << b;
+        }
+        const uint32_t hot = live ? (gt | eq) : 0u;
+        s_hot[w] = hot;
+        if (live) job.hotmap[((uint64_t)d * G.r + i) * rw + word] = hot;
+        uint32_t z = live ? 32u * G.g - ones : 0u, nh = (uint32_t)__popc(hot);
+        constexpr uint32_t mask = W == 32 ? 0xFFFFFFFFu : (1u << W) - 1u;
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) {
+            z += __shfl_xor_sync(mask, z, o);
+            nh += __shfl_xor_sync(mask, nh, o);
+        }
+        __threadfence();  // every lane's bitmap word, before the row's count
+        __syncwarp(mask);
+        if (w == 0) {
+            atomicAdd(&job.st->zr[d][i], (unsigned long long)z);
+            if (nh) atomicAdd(&job.st->nhot[d][i], nh);
+            s_list = i < 2 && atomicAdd(&job.st->rows_done[d][i], 1u) == wgroups - 1;
+        }
+    }
+    __syncthreads();
+    const uint32_t hot = s_hot[w];
+    if (hot) {
+        uint32_t x[32];
+        const uint32_t *p = opaque(src);
+#pragma unroll
+        for (uint32_t j = 0; j < 32; j++, p += ps) x[j] = __ldcg(p);
+        transpose32_regs(x);  // x[b]: word tt of estimator 32 word + b
+        uint32_t *dst = job.grid + (uint64_t)d * G.dir_words + (uint64_t)i * G.row_words + (uint64_t)(32u * word) * TC + tt;
+#pragma unroll
+        for (uint32_t b = 0; b < 32; b++)
+            if (hot >> b & 1u) dst[b * TC] = x[b];
+    }
+    if (any) {
+        uint32_t *p = opaque(src);
+#pragma unroll
+        for (uint32_t j = 0; j < 32; j++, p += ps)
+            if (any >> j & 1u) *p = 0u;
+    }
+    if (s_list) {
+        __threadfence();
+        list_hot(job.hotmap + ((uint64_t)d * G.r + i) * rw, rw, job.he + ((uint64_t)d * 2 + i) * (1ull << G.k));
+    }
+}
+
+cudaError_t launch_plane_scan(const FoldJob &one, const FoldJob *jobs, uint32_t njobs, const Geometry &G, uint32_t ps,
+                              cudaStream_t s) {
+    if (jobs && njobs == 0) return cudaSuccess;
+    if (!fold_stats_fit(G)) return cudaErrorInvalidValue;
+    const uint32_t W = kScanThreads / G.wpc, rw = (1u << G.k) >> 5;
+    const uint64_t blocks = (uint64_t)(jobs ? njobs : 1u) * G.dirs * G.r * ((rw + W - 1) / W);
+    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    switch (G.wpc) {
+        case 8: k_plane_scan<8><<<(unsigned)blocks, kScanThreads, 0, s>>>(one, jobs, G, ps); break;
+        case 16: k_plane_scan<16><<<(unsigned)blocks, kScanThreads, 0, s>>>(one, jobs, G, ps); break;
+        case 32: k_plane_scan<32><<<(unsigned)blocks, kScanThreads, 0, s>>>(one, jobs, G, ps); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 }  // namespace sd
