@@ -701,6 +701,19 @@ static int ensure_plane_bins(sd_handle *owner, uint64_t words) {
     return SD_OK;
 }
 
+// Whether a round of m pairs over G's directions, short of the tuning's full
+// round, sets its bits in the plane copy directly (k_plane_direct).  Both
+// sides measured on GB300: a direct round takes 6 us and 1 us per 180,000
+// bit-sets while the plane copy fits L2; a binned one at least 22 us and
+// 0.5 us per MiB of plane copy, which every round sweeps.  They meet at
+// 3 M bit-sets (2^20 pairs of a 0.5 MiB copy: 27 and 26 us) to 6 M (2^19.5
+// pairs of a 32 MiB copy: 33 and 37 us), and for a copy beyond L2 at 8 M to
+// 16 M (2^20 pairs of 256 MiB: 78 and 155 us; 2^21: 258 and 164 us).
+static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
+    const uint64_t copy_words = (uint64_t)G.dirs * G.g * plane_words(G);
+    return m < round && m * G.dirs * G.r <= std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3);
+}
+
 // Algorithm 1 binned by plane over n device pairs of h, in rounds of at
 // most `round` pairs through `bins` (bin_words of them, at least the bins
 // of one round), on stream s; failures are reported on `rep`.  A round
@@ -721,11 +734,16 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
         P.nbins = h->G.g;
         P.planes += (uint64_t)dir * h->G.g * P.ps;
     }
-    if (plane_bin_words(G, std::min(round, n)) > bin_words)
+    if (!plane_direct(G, n, round) && plane_bin_words(G, std::min(round, n)) > bin_words)
         return rep->fail(SD_ERR_ARG, "plane update: %llu bin words for rounds of %llu pairs",
                          (unsigned long long)bin_words, (unsigned long long)round);
     for (uint64_t off = 0; off < n; off += round) {
         const uint64_t m = std::min(round, n - off);
+        if (plane_direct(G, m, round)) {
+            SD_CK(rep, launch_plane_direct(pairs + 2 * off, m, G, P, h->num_sms, s));
+            launched(1);
+            continue;
+        }
         const uint64_t prev = h->plane_layout_view == dir ? h->plane_prev_pairs : 0;
         PlaneLayout L = kLayoutCount;
         if (prev && m <= prev && plane_bin_words(G, prev) <= bin_words) L = kLayoutReuse;
@@ -779,7 +797,8 @@ static int update_device(sd_handle *h, const uint32_t *pairs, uint64_t n, int di
         int rc = ensure_plane_state(h);
         if (rc != SD_OK) return rc;
         const uint64_t round = 1ull << h->T.plane_round_log2;
-        rc = ensure_plane_bins(h, plane_bin_words(h->G, round));
+        if (!plane_direct(G, n, round))
+            rc = ensure_plane_bins(h, plane_bin_words(h->G, round));
         if (rc != SD_OK) return rc;
         return plane_rounds(h, pairs, n, dir, h->plane_bins, h->plane_bins_words, round, h->stream, h);
     }

@@ -271,6 +271,9 @@ size_t plane_bin_smem_bytes(uint32_t tile_pairs, uint32_t dirs, uint32_t nbins);
 enum PlaneLayout { kLayoutReuse = 0, kLayoutScale = 1, kLayoutCount = 2 };
 cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
                                cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs);
+// a short round without bins: the n pairs' bits ORed into the plane copy in place
+cudaError_t launch_plane_direct(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
+                                cudaStream_t s);
 // dst = OR of `count` arrays of `words` words at src (words a multiple of 4)
 cudaError_t launch_or_words(uint32_t *dst, const uint32_t *src, uint64_t words, uint32_t count, int num_sms,
                             cudaStream_t s);

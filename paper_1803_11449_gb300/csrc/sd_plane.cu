@@ -501,6 +501,46 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
     write_layout(P, true, s_warp);
 }
 
+// ----------------------------------------------------------------- direct
+// A short round: every key's bits ORed into the plane copy where they lie,
+// one pair per thread, with no bins and no planes in shared memory.  Bound
+// by the L2's random reductions; the binned round's floor is the sweep of
+// the whole plane copy through shared memory, whatever the pairs.  A pair
+// equal to its predecessor (a flow's packets in a burst) is skipped.
+template <int DIRS>
+__global__ void __launch_bounds__(256)
+k_plane_direct(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArgs P) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const bool pair8 = ((uintptr_t)pairs & 7u) == 0;
+    for (uint64_t p0 = (uint64_t)blockIdx.x * blockDim.x; p0 < n; p0 += stride) {
+        const uint64_t p = p0 + threadIdx.x;
+        const bool ok = p < n;
+        uint32_t s = 0, t = 0;
+        if (ok && pair8) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(pairs) + p);
+            s = v.x;
+            t = v.y;
+        } else if (ok) {
+            s = ld_stream_u32(pairs + 2 * p);
+            t = ld_stream_u32(pairs + 2 * p + 1);
+        }
+        const uint32_t us = __shfl_up_sync(0xFFFFFFFFu, s, 1), ut = __shfl_up_sync(0xFFFFFFFFu, t, 1);
+        if (!ok || ((threadIdx.x & 31u) && us == s && ut == t)) continue;
+        set_key_bits<DIRS>(G, P, h1v(G.h[0].A1, G.h[0].B1, G.lg, t), s);
+        if (DIRS == 2) set_key_bits<DIRS>(G, P, G.g + h1v(G.h[1].A1, G.h[1].B1, G.lg, s), t);
+    }
+}
+
+cudaError_t launch_plane_direct(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
+                                cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    auto kern = G.dirs == 2 ? k_plane_direct<2> : k_plane_direct<1>;
+    uint64_t blocks = (n + 255) / 256;
+    if (blocks > (uint64_t)num_sms * 32) blocks = (uint64_t)num_sms * 32;
+    kern<<<(unsigned)blocks, 256, 0, s>>>(pairs, n, G, P);
+    return cudaGetLastError();
+}
+
 // --------------------------------------------------------------- launchers
 size_t plane_bin_smem_bytes(uint32_t tile_pairs, uint32_t dirs, uint32_t nbins) {
     return (size_t)dirs * tile_pairs * 8 + (size_t)nbins * 16;
