@@ -148,6 +148,7 @@ struct CloseState {
     double psi[2];
     uint64_t nh[2];                        // hits per direction
     const unsigned long long *keys[2];     // their sorted keys in pinned host memory
+    bool queued_b;                         // phase B queued work
 };
 
 // The report's hits: a plain growable array that is not zero-filled when it
@@ -198,7 +199,8 @@ struct sd_handle {
     uint32_t *cand = nullptr;          // [dirs][cand_cap]
     unsigned long long *hits = nullptr;   // [dirs][hits_cap]
     unsigned long long *hits_tmp = nullptr;  // [dirs][hits_cap]: scratch of the large-list sort
-    unsigned long long *hits_h = nullptr; // pinned [dirs][kSortSmall]
+    unsigned long long *hits_h = nullptr; // pinned [2][finish_cap]: ordered hits
+    uint64_t finish_cap = 0;
     uint64_t cand_cap = 0, hits_cap = 0, report_cap = 0, pair_cap = 0;
     unsigned long long *big_h = nullptr;  // pinned [2][hits_cap]: large sorted hit lists
     void *ss_d = nullptr;                 // [2] sample-sort scratch (kSampleScratchBytes each)
@@ -215,7 +217,7 @@ struct sd_handle {
     CloseJob *cj_d = nullptr, *cj_h = nullptr;  // cj_h pinned
     StatBlock *cb_st_d = nullptr, *cb_st_h = nullptr;
     unsigned long long *cb_hits_d = nullptr, *cb_hits_h = nullptr;
-    unsigned long long *cb_base_d = nullptr, *cb_base_h = nullptr;  // tile and candidate offsets
+    unsigned long long *cb_base_d = nullptr, *cb_base_h = nullptr;  // tile offsets
     FoldJob *fj_d = nullptr, *fj_h = nullptr;  // members' plane folds (fj_h pinned)
     uint32_t cj_cap = 0;
 
@@ -395,7 +397,7 @@ static void resolve_caps(const sd_params *p, uint64_t *pair_cap, uint64_t *cand_
                          uint64_t *report_cap, uint64_t *stage) {
     *pair_cap = p->pair_cap ? p->pair_cap : (1ull << 32);
     *cand_cap = p->cand_cap ? p->cand_cap : (1ull << 20);
-    *hits_cap = next_pow2(*cand_cap);
+    *hits_cap = std::max<uint64_t>(2, next_pow2(*cand_cap));  // (lists start on 16 bytes)
     *report_cap = p->report_cap ? p->report_cap : (uint64_t)p->dirs * *cand_cap;
     // host-ingest chunks: 2^22 pairs keep the last chunk's kernels short; a
     // DHLA larger than L2 takes 2^24 (each chunk is one binning round, and
@@ -560,7 +562,8 @@ static int create_impl(const sd_params *p, sd_handle *h) {
     SD_CK(h, cudaMalloc(&h->hits, (uint64_t)p->dirs * h->hits_cap * 8));
     SD_CK(h, cudaMalloc(&h->hits_tmp, (uint64_t)p->dirs * h->hits_cap * 8));
     SD_CK(h, cudaMallocHost(&h->st_h, sizeof(StatBlock)));
-    SD_CK(h, cudaMallocHost(&h->hits_h, (uint64_t)2 * kSortSmall * 8));
+    h->finish_cap = kSortSmall;
+    SD_CK(h, cudaMallocHost(&h->hits_h, (uint64_t)2 * h->finish_cap * 8));
     SD_CK(h, launch_reset(h->grid, words, h->st_d, h->num_sms, h->stream));
     SD_CK(h, cudaStreamSynchronize(h->stream));
     h->grid_clean = true;
@@ -1247,11 +1250,39 @@ struct CloseTrace {
 // GPU work and share host synchronisations (sd_close_many).  Each phase only
 // queues work on the handle's stream; the caller synchronises the stream
 // between phases.
-//   A: hot estimators and row statistics (Algorithm 2, first loop; §4.2)
-//   B: host decisions (psi, szmax, caps), then restore K, estimate SZ,
-//      order small hit lists (Algorithm 2 / Algorithms 3-4, §4.2)
+//   A: hot estimators and row statistics (Algorithm 2, first loop; §4.2),
+//      and with the default restore all of K, SZ and the ordered hits behind
+//      them: the kernels take the directions that run and a bound on SZ from
+//      the statistics themselves, so the host is not waited for in between
+//      (a round trip and four copies less: 12 to 20 us of a close)
+//   B: host decisions (psi, szmax, caps); with the staged join, then restore
+//      K, estimate SZ, order small hit lists (Algorithms 3-4, §4.2)
 //   C: order the large hit lists
 //   D: build the report (Eq. 4), clear the DHLA for the next window
+static void restore_buffers(sd_handle *h, RestoreArgs &A) {
+    A.grid = h->grid;
+    A.he = h->he;
+    A.hotmap = h->hotmap;
+    A.cand = h->cand;
+    A.hits = h->hits;
+    A.stats = h->st_d;
+    A.cand_cap = h->cand_cap;
+    A.hits_cap = h->hits_cap;
+}
+
+// Restore, SZ and the ordered hits from the row statistics in st_d; the hits
+// and the StatBlock end in hits_h and st_h.
+static int queue_restore(sd_handle *h, float xfac) {
+    RestoreArgs A;
+    std::memset(&A, 0, sizeof A);
+    restore_buffers(h, A);
+    SD_CK(h, launch_restore(h->G, A, h->pair_cap, xfac, h->num_sms, h->stream));
+    SD_CK(h, launch_close_finish(h->hits, h->hits_cap, h->st_d, h->hits_h, h->finish_cap, h->hits_tmp,
+                                 h->st_h, h->G.dirs, h->stream));
+    launched(2);
+    return SD_OK;
+}
+
 static int close_phase_a(sd_handle *h, sd_report *out) {
     std::memset(out, 0, sizeof *out);
     std::memset(&h->cs, 0, sizeof h->cs);
@@ -1282,6 +1313,7 @@ static int close_phase_a(sd_handle *h, sd_report *out) {
         SD_CK(h, launch_compact(h->hotmap, h->G, h->he, 2, h->stream));
         launched(1);
     }
+    if (h->T.restore == 0) return queue_restore(h, (float)std::exp(-h->p.theta / (double)h->G.g));
     SD_CK(h, cudaMemcpyAsync(h->st_h, h->st_d, sizeof(StatBlock), cudaMemcpyDeviceToHost, h->stream));
     return SD_OK;
 }
@@ -1323,14 +1355,7 @@ static bool close_decide(sd_handle *h, sd_report *out) {
         A.n1[d] = (uint32_t)n1;
         A.szmax[d] = szmax;
     }
-    A.grid = h->grid;
-    A.he = h->he;
-    A.hotmap = h->hotmap;
-    A.cand = h->cand;
-    A.hits = h->hits;
-    A.stats = h->st_d;
-    A.cand_cap = h->cand_cap;
-    A.hits_cap = h->hits_cap;
+    restore_buffers(h, A);
     return A.run[0] || A.run[1];
 }
 
@@ -1338,6 +1363,7 @@ static int close_phase_b(sd_handle *h, sd_report *out) {
     if (!close_decide(h, out)) return SD_OK;
     const Geometry &G = h->G;
     RestoreArgs &A = h->cs.A;
+    h->cs.queued_b = h->T.restore == 1;
     if (h->T.restore == 1) {
         if (!h->jsub) {
             h->join_cap = 4 * h->cand_cap;
@@ -1361,8 +1387,17 @@ static int close_phase_b(sd_handle *h, sd_report *out) {
         SD_CK(h, launch_join(G, J, h->num_sms, h->stream));
         launched(1 + (G.r - 2));
     } else {
-        SD_CK(h, launch_restore(G, A, h->num_sms, h->stream));
-        launched(((A.run[0] && A.n0[0] && A.n1[0]) || (A.run[1] && A.n0[1] && A.n1[1])) ? 1 : 0);
+        // done in phase A; the SZ bound that the kernels used covers szmax by
+        // far more than its rounding (see szmax_bound), else once more without one
+        bool short_of = false;
+        for (uint32_t d = 0; d < G.dirs; d++)
+            short_of = short_of || (A.run[d] && A.n0[d] && A.n1[d] && A.szmax[d] > h->st_h->szmax_used[d]);
+        if (!short_of) return SD_OK;
+        h->cs.queued_b = true;
+        for (uint32_t d = 0; d < 2; d++) h->st_h->ncand[d] = h->st_h->nhits[d] = h->st_h->big_sort[d] = 0;
+        h->st_h->finish_done = 0;
+        SD_CK(h, cudaMemcpyAsync(h->st_d, h->st_h, sizeof(StatBlock), cudaMemcpyHostToDevice, h->stream));
+        return queue_restore(h, 1e4f);
     }
     SD_CK(h, launch_estimate(G, A, h->num_sms, h->stream));
     SD_CK(h, launch_sort_small(h->hits, h->hits_cap, h->st_d, A.run, G.dirs, h->stream));
@@ -1370,7 +1405,7 @@ static int close_phase_b(sd_handle *h, sd_report *out) {
     SD_CK(h, cudaMemcpyAsync(h->st_h, h->st_d, sizeof(StatBlock), cudaMemcpyDeviceToHost, h->stream));
     for (uint32_t d = 0; d < G.dirs; d++)
         if (A.run[d])
-            SD_CK(h, cudaMemcpyAsync(h->hits_h + (uint64_t)d * kSortSmall, h->hits + (uint64_t)d * h->hits_cap,
+            SD_CK(h, cudaMemcpyAsync(h->hits_h + (uint64_t)d * h->finish_cap, h->hits + (uint64_t)d * h->hits_cap,
                                      std::min<uint64_t>(kSortSmall, h->hits_cap) * 8, cudaMemcpyDeviceToHost,
                                      h->stream));
     return SD_OK;
@@ -1381,6 +1416,23 @@ static int close_phase_c(sd_handle *h, sd_report *out, bool *need_sync) {
     CloseState &c = h->cs;
     *need_sync = false;
     h->ss_check[0] = h->ss_check[1] = false;
+    // lists that were ordered but did not fit hits_h: a larger one, for this
+    // close and the next ones (any list already in the old one moves along)
+    uint64_t want = 0;
+    for (uint32_t d = 0; d < h->G.dirs; d++)
+        if (c.A.run[d] && h->st_h->big_sort[d] == 2) want = std::max<uint64_t>(want, h->st_h->nhits[d]);
+    if (want > h->finish_cap) {
+        const uint64_t cap = next_pow2(want);
+        unsigned long long *grown = nullptr;
+        SD_CK(h, cudaMallocHost(&grown, (uint64_t)2 * cap * 8));
+        for (uint32_t d = 0; d < h->G.dirs; d++)
+            if (c.A.run[d] && h->st_h->big_sort[d] == 0)
+                std::memcpy(grown + d * cap, h->hits_h + d * h->finish_cap,
+                            std::min<uint64_t>(h->st_h->nhits[d], h->finish_cap) * 8);
+        cudaFreeHost(h->hits_h);
+        h->hits_h = grown;
+        h->finish_cap = cap;
+    }
     for (uint32_t d = 0; d < h->G.dirs; d++) {
         if (!c.A.run[d]) continue;
         const uint64_t nk = h->st_h->ncand[d];
@@ -1398,8 +1450,14 @@ static int close_phase_c(sd_handle *h, sd_report *out, bool *need_sync) {
             continue;
         }
         c.nh[d] = h->st_h->nhits[d];
-        c.keys[d] = h->hits_h + (uint64_t)d * kSortSmall;
+        c.keys[d] = h->hits_h + (uint64_t)d * h->finish_cap;
         if (!h->st_h->big_sort[d]) continue;
+        if (h->st_h->big_sort[d] == 2) {
+            SD_CK(h, cudaMemcpyAsync(h->hits_h + (uint64_t)d * h->finish_cap, h->hits_tmp + (uint64_t)d * h->hits_cap,
+                                     c.nh[d] * 8, cudaMemcpyDeviceToHost, h->stream));
+            *need_sync = true;
+            continue;
+        }
         unsigned long long *sorted = nullptr;
         uint32_t *overflow = nullptr;
         int nl = 0;
@@ -1465,21 +1523,26 @@ static int close_phase_d(sd_handle *h, sd_report *out, bool reset = true) {
         sd_hit *out_h = h->report.data() + at;
         const double *t = tbl.data();
         const size_t tn = tbl.size();
+        size_t kept = 0;
         for (uint64_t q = 0; q < nh; q++) {
             const unsigned long long key = keys[q];
             const uint32_t sz = (uint32_t)(key & 0xFFFFFFFFull);
-            out_h[q].ip = (uint32_t)(key >> 32);
-            out_h[q].sz = sz;
-            out_h[q].dir = d;
-            out_h[q].reserved = 0;
-            out_h[q].est = sz < tn ? t[sz] : eq4(G.g, G.r, c.psi[d], sz);
+            if (sz >= tn) continue;  // above szmax: within the kernels' bound only
+            out_h[kept].ip = (uint32_t)(key >> 32);
+            out_h[kept].sz = sz;
+            out_h[kept].dir = d;
+            out_h[kept].reserved = 0;
+            out_h[kept].est = t[sz];
+            kept++;
         }
+        h->report.truncate(at + kept);
     }
     h->have_close = true;
     // clear the DHLA and the counters for the next window (stream-ordered;
     // a batched close clears all its handles in one launch instead)
     if (reset && h->grid_stale) {
-        SD_CK(h, cudaMemsetAsync(h->st_d, 0, sizeof(StatBlock), h->stream));
+        if (h->T.restore != 0)  // (else k_close_finish has cleared it)
+            SD_CK(h, cudaMemsetAsync(h->st_d, 0, sizeof(StatBlock), h->stream));
     } else if (reset) {
         SD_CK(h, launch_reset(h->grid, (uint64_t)G.dirs * G.dir_words, h->st_d, h->num_sms, h->stream));
         launched(1);
@@ -1535,7 +1598,7 @@ int sd_close_window(sd_handle *h, sd_report *out) {
     trace.mark(0);
     rc = close_phase_b(h, out);
     if (rc != SD_OK) return rc;
-    SD_CK(h, cudaStreamSynchronize(h->stream));
+    if (h->cs.queued_b) SD_CK(h, cudaStreamSynchronize(h->stream));
     trace.mark(1);
     bool big = false;
     rc = close_phase_c(h, out, &big);
@@ -1594,8 +1657,8 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         SD_CK(d, cudaMallocHost(&d->cb_st_h, count * sizeof(StatBlock)));
         SD_CK(d, cudaMalloc(&d->cb_hits_d, (uint64_t)count * 2 * kSortSmall * 8));
         SD_CK(d, cudaMallocHost(&d->cb_hits_h, (uint64_t)count * 2 * kSortSmall * 8));
-        // tile offsets (device + host) and candidate offsets (device), 2 count + 1 each
-        SD_CK(d, cudaMalloc(&d->cb_base_d, (uint64_t)2 * (2 * count + 1) * 8));
+        // tile offsets, 2 count + 1
+        SD_CK(d, cudaMalloc(&d->cb_base_d, (uint64_t)(2 * count + 1) * 8));
         SD_CK(d, cudaMallocHost(&d->cb_base_h, (uint64_t)(2 * count + 1) * 8));
         SD_CK(d, cudaMalloc(&d->fj_d, count * sizeof(FoldJob)));
         SD_CK(d, cudaMallocHost(&d->fj_h, count * sizeof(FoldJob)));
@@ -1698,8 +1761,7 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
     if (any) {
         SD_CK(d, cudaMemcpyAsync(d->cj_d, d->cj_h, count * sizeof(CloseJob), cudaMemcpyHostToDevice, s));
         int nl = 0;
-        SD_CK(d, launch_restore_many(d->cj_d, d->cj_h, count, d->cb_base_d, d->cb_base_h,
-                                     d->cb_base_d + (2 * count + 1), d->num_sms, s, &nl));
+        SD_CK(d, launch_restore_many(d->cj_d, d->cj_h, count, d->cb_base_d, d->cb_base_h, d->num_sms, s, &nl));
         SD_CK(d, launch_gather_many(d->cj_d, count, d->cb_st_d, d->cb_hits_d, s));
         launched(nl + 1);
         SD_CK(d, cudaMemcpyAsync(d->cb_st_h, d->cb_st_d, count * sizeof(StatBlock), cudaMemcpyDeviceToHost, s));
@@ -1718,7 +1780,7 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         bool b = false;
         rcs[i] = close_phase_c(h, &outs[i], &b);
         for (uint32_t dd = 0; dd < G.dirs; dd++)
-            if (h->cs.keys[dd] == h->hits_h + (uint64_t)dd * kSortSmall)
+            if (h->cs.keys[dd] == h->hits_h + (uint64_t)dd * h->finish_cap)
                 h->cs.keys[dd] = d->cb_hits_h + ((uint64_t)i * 2 + dd) * kSortSmall;
         big[i] = b;
         any_big = any_big || b;

@@ -6,11 +6,14 @@
 //                 |HE(i)|.
 //   k_compact     sorted lists HE(0) and HE(1) (all HE(i) for the staged
 //                 join of sd_join.cu) from their bitmaps.
-//   k_restore     the candidate set K = {a : DH_i(a) in HE(i) for all i}.
-//   k_estimate    SZ(a) from ULE(a) = AND of a's r estimators (16-byte
+//   k_restore     the candidate set K = {a : DH_i(a) in HE(i) for all i},
+//                 and SZ(a) from ULE(a) = AND of a's r estimators (16-byte
 //                 chunks, several candidates per warp), keeping (a, SZ) when
 //                 SZ <= szmax.
-//   k_sort_small  orders each direction's hits by address (bitonic, smem).
+//   k_close_finish  each direction's hits ordered by address, with the
+//                 counters, into host memory.
+//   k_estimate, k_sort_small  SZ of a K made by the staged join, and its hits
+//                 ordered (bitonic, smem).
 //   k_ss_*        the same for up to 2^19 hits: a sample sort (splitters
 //                 from a sorted sample, keys scattered to buckets, each
 //                 bucket sorted by one block).
@@ -160,22 +163,10 @@ __device__ __forceinline__ bool hot_at(const uint32_t *bm_row, uint32_t c) {
 
 constexpr uint32_t kRestoreTileMax = 256;  // c0 values per k_restore tile
 
-// Per-warp output buffers of k_restore: candidates and hits are reserved in
-// the global lists 32 at a time (one atomic per flush instead of one per
-// finding warp, which serialised on the two counters).
+// Per-warp output buffers of the restore: candidates and hits are reserved
+// in the global lists 32 or more at a time (one atomic per flush instead of
+// one per finding warp, which serialised on the two counters).
 constexpr int kWarpBuf = 64;
-
-__device__ __forceinline__ void flush_cands(const RestoreArgs &A, uint32_t dir, uint32_t *cbuf, uint32_t &ccount,
-                                            uint32_t lane) {
-    if (ccount == 0) return;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(&A.stats->ncand[dir], (unsigned long long)ccount);
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    for (uint32_t q = lane; q < ccount; q += 32)
-        if (base + q < A.cand_cap) A.cand[(uint64_t)dir * A.cand_cap + base + q] = cbuf[q];
-    ccount = 0;
-    __syncwarp();
-}
 
 __device__ __forceinline__ void flush_hits(const RestoreArgs &A, uint32_t dir, unsigned long long *hbuf,
                                            uint32_t &hcount, uint32_t lane) {
@@ -189,6 +180,72 @@ __device__ __forceinline__ void flush_hits(const RestoreArgs &A, uint32_t dir, u
     __syncwarp();
 }
 
+// SZ of n <= kWarpBuf candidates in x[] (shared memory) by one warp: the zero
+// bits of ULE(a), the AND of a's r estimators; those with SZ <= szmax go to
+// the hit list.  lpc lanes per candidate, each ANDing 16-byte chunks (4-byte
+// words for g < 128) of the r estimators.
+__device__ __forceinline__ void estimate_warp(const Geometry &G, const RestoreArgs &A, uint32_t dir, int szmax,
+                                              const uint32_t *x_of, uint32_t n, unsigned long long *hbuf,
+                                              uint32_t lane) {
+    const uint32_t A0 = dir ? G.h[1].A0 : G.h[0].A0;
+    const uint32_t *gdir = A.grid + (uint64_t)dir * G.dir_words;
+    const uint32_t kmask = (1u << G.k) - 1u;
+    const bool wide = G.wpc >= 4;
+    const uint32_t chunks = wide ? G.wpc >> 2 : G.wpc;
+    const uint32_t lpc = chunks < 32u ? chunks : 32u;
+    const uint32_t cpw = 32u / lpc, sub = lane / lpc, sl = lane % lpc;
+    uint32_t hcount = 0;
+    for (uint32_t q0 = 0; q0 < n; q0 += cpw) {
+        const uint32_t q = q0 + sub;
+        const bool ok = q < n;
+        const uint32_t x = ok ? x_of[q] : 0u;
+        const uint32_t c0 = dh0(A0, G.k, x);
+        uint32_t ones = 0;
+        if (ok) {
+            for (uint32_t c = sl; c < chunks; c += lpc) {
+                uint4 ule = make_uint4(~0u, wide ? ~0u : 0u, wide ? ~0u : 0u, wide ? ~0u : 0u);
+#pragma unroll
+                for (uint32_t i = 0; i < 8; i++) {
+                    if (i >= G.r) break;
+                    const uint32_t ci = i == 0 ? c0 : ((shr_clamp(x, (i - 1u) * G.alpha) & kmask) ^ c0);
+                    const uint32_t *cell = gdir + (uint64_t)i * G.row_words + (uint64_t)ci * G.wpc;
+                    if (wide) {
+                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(cell) + c);
+                        ule.x &= v.x; ule.y &= v.y; ule.z &= v.z; ule.w &= v.w;
+                    } else {
+                        ule.x &= __ldg(cell + c);
+                    }
+                }
+                ones += __popc(ule.x) + __popc(ule.y) + __popc(ule.z) + __popc(ule.w);
+            }
+        }
+        for (uint32_t o = lpc >> 1; o > 0; o >>= 1) ones += __shfl_xor_sync(0xFFFFFFFFu, ones, o);
+        const bool hit = ok && sl == 0 && (int)(G.g - ones) <= szmax;
+        const unsigned hb = __ballot_sync(0xFFFFFFFFu, hit);
+        if (hit) hbuf[hcount + __popc(hb & ((1u << lane) - 1u))] = ((unsigned long long)x << 32) | (G.g - ones);
+        hcount += __popc(hb);
+    }
+    __syncwarp();
+    flush_hits(A, dir, hbuf, hcount, lane);
+}
+
+// A warp's buffered candidates to K, and their SZ and hits at once (the
+// estimators are hot, so in the DHLA; the loads hide behind other warps'
+// tests).  Hits of a direction whose K overflows are dropped by the host.
+__device__ __forceinline__ void flush_cands(const Geometry &G, const RestoreArgs &A, uint32_t dir, int szmax,
+                                            uint32_t *cbuf, unsigned long long *hbuf, uint32_t &ccount,
+                                            uint32_t lane) {
+    if (ccount == 0) return;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(&A.stats->ncand[dir], (unsigned long long)ccount);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    for (uint32_t q = lane; q < ccount; q += 32)
+        if (base + q < A.cand_cap) A.cand[(uint64_t)dir * A.cand_cap + base + q] = cbuf[q];
+    if (base < A.cand_cap) estimate_warp(G, A, dir, szmax, cbuf, ccount, hbuf, lane);
+    ccount = 0;
+    __syncwarp();
+}
+
 // 32-bit load from shared memory at byte address `addr`.
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     uint32_t v;
@@ -196,301 +253,311 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     return v;
 }
 
-// One (c0, c1) test for k >= 16 and R rows, the hot bitmap rows 2..R-1 in
-// shared memory at byte address hot2s (row i - 2 at + (i - 2) nw 4): a's low
-// k bits are L = c0 ^ c1; its high 32 - k bits are A0^-1 (c0 >> (2k - 32) -
-// (A0 L >> k)) mod 2^(32-k), computed as one multiply by A0^-1 2^k; unless
-// k = 16, the low 2k - 32 bits of c0 must also match the top bits of A0 L
-// mod 2^k.  Returns whether a is in K; a is set.
-template <int R, bool K16, int ALPHA>
-__device__ __forceinline__ bool restore_test(uint32_t c0, uint32_t c1, uint32_t k, uint32_t kmask, uint32_t lowbits,
-                                             uint32_t lowmask, uint32_t A0, uint32_t A0inv_k, uint32_t hot2s,
-                                             uint32_t nw4, const uint32_t (&sh)[R > 2 ? R - 2 : 1], uint32_t &a) {
-    const uint32_t L = c0 ^ c1;
-    const uint32_t Q = A0 * L;
-    uint32_t found = 1u;
-    if (K16) {
-        a = A0inv_k * (c0 - (Q >> 16)) + L;
-    } else {
-        a = A0inv_k * ((c0 >> lowbits) - (Q >> k)) + L;
-        found = ((Q & kmask) >> (32u - k)) == (c0 & lowmask);
-    }
-#pragma unroll
-    for (int i = 2; i < R; i++) {
-        // with k = 16 and a compile-time alpha the shifts and masks are constants
-        const uint32_t s = ALPHA ? (uint32_t)((i - 1) * ALPHA) : sh[i - 2];
-        const uint32_t m = K16 ? 0xFFFFu : kmask;
-        const uint32_t ci = (ALPHA && s >= 32u ? 0u : (ALPHA ? (a >> (s & 31u)) : shr_clamp(a, s))) & m ^ c0;
-        const uint32_t word = lds_u32(hot2s + (uint32_t)(i - 2) * nw4 + ((ci >> 3) & ~3u));
-        found &= word >> (ci & 31u);
-    }
-    return found & 1u;
+// How the high 32 - k bits of an address follow from (c0, c1): below k = 16
+// each t < 2^(32-2k) is one, at 16 there is exactly one, above 16 at most one.
+enum RestoreBits { kBelow16 = 0, kIs16 = 1, kAbove16 = 2 };
+
+// What a test needs besides c0, c1 and t.
+struct RestoreConsts {
+    uint32_t k, kmask, lowbits, lowmask, ulog, A0, A0inv_k, nw, alpha;
+    uint32_t hot2s;        // rows 2.. of the hot bitmap in shared memory (byte address)
+    const uint32_t *hot2;  // and in global memory
+};
+
+// bit `ci` of row i (>= 2) of the hot bitmap
+template <bool SMEM>
+__device__ __forceinline__ uint32_t hot_bit(const RestoreConsts &C, uint32_t i, uint32_t ci) {
+    const uint32_t w = SMEM ? lds_u32(C.hot2s + (i - 2u) * C.nw * 4u + ((ci >> 3) & ~3u))
+                            : __ldcg(C.hot2 + (uint64_t)(i - 2u) * C.nw + (ci >> 5));
+    return w >> (ci & 31u) & 1u;
 }
 
-// The tests of two c1 values per thread against the tile's c0 values, for
-// k >= 16 with the hot bitmap in shared memory; candidates go to the warp's
-// buffer.
-template <int R, bool K16, int ALPHA>
-__device__ __forceinline__ void restore_c1x2(const Geometry &G, const RestoreArgs &A, uint32_t dir,
-                                             const uint32_t *s_c0, uint32_t nc0, uint32_t hot2s, uint32_t nw,
-                                             uint32_t c1a, bool va, uint32_t c1b, bool vb, uint32_t A0,
-                                             uint32_t A0inv, uint32_t *cbuf, uint32_t &ccount, uint32_t lane) {
-    const uint32_t k = G.k, kmask = (1u << k) - 1u;
-    const uint32_t lowbits = 2u * k - 32u, lowmask = (1u << lowbits) - 1u;
-    const uint32_t A0inv_k = A0inv << k, nw4 = nw * 4u;
-    uint32_t sh[R > 2 ? R - 2 : 1];
+// Whether a is hot in rows FROM .. R-1 (with k = 16 and a compile-time alpha
+// the shifts and masks are constants).
+template <int FROM, int R, int KM, int ALPHA, bool SMEM>
+__device__ __forceinline__ bool rows_hot(const RestoreConsts &C, uint32_t a, uint32_t c0) {
+    uint32_t found = 1u;
 #pragma unroll
-    for (int i = 2; i < R; i++) sh[i - 2] = (uint32_t)(i - 1) * G.alpha;
+    for (int i = FROM; i < R; i++) {
+        const uint32_t s = ALPHA ? (uint32_t)((i - 1) * ALPHA) : (uint32_t)(i - 1) * C.alpha;
+        const uint32_t m = KM == kIs16 ? 0xFFFFu : C.kmask;
+        const uint32_t ci = (ALPHA && s >= 32u ? 0u : (ALPHA ? (a >> (s & 31u)) : shr_clamp(a, s))) & m ^ c0;
+        if (SMEM) found &= hot_bit<true>(C, i, ci);
+        else if (found) found &= hot_bit<false>(C, i, ci);
+    }
+    return found;
+}
+
+// The first stage of one (c0, c1, t) test: a's low k bits are L = c0 ^ c1;
+// its high 32 - k bits are A0^-1 (u - (A0 L >> k)) mod 2^(32-k), computed as
+// one multiply by A0^-1 2^k, with u = c0 << (32-2k) | t below k = 16 and
+// c0 >> (2k-32) from there on.  For k > 16 the low 2k - 32 bits of c0 must
+// match the top bits of A0 L mod 2^k (one pair in 2^(2k-32) does); otherwise
+// a's row 2 must be hot.
+template <int R, int KM, int ALPHA, bool SMEM>
+__device__ __forceinline__ bool restore_first(const RestoreConsts &C, uint32_t c0, uint32_t c1, uint32_t t,
+                                              uint32_t &a) {
+    const uint32_t L = c0 ^ c1;
+    const uint32_t Q = C.A0 * L;
+    if (KM == kIs16) a = C.A0inv_k * (c0 - (Q >> 16)) + L;
+    else if (KM == kBelow16) a = C.A0inv_k * (((c0 << C.ulog) | t) - (Q >> C.k)) + L;
+    else a = C.A0inv_k * ((c0 >> C.lowbits) - (Q >> C.k)) + L;
+    if (KM == kAbove16) return ((Q & C.kmask) >> (32u - C.k)) == (c0 & C.lowmask);
+    return rows_hot<2, 3, KM, ALPHA, SMEM>(C, a, c0);
+}
+
+// Per-warp buffers of a block's restore.
+struct WarpBufs {
+    uint2 *queue;              // [96] (a, c0) that passed the first stage
+    uint32_t *cand;            // [kWarpBuf] members of K
+    unsigned long long *hits;  // [kWarpBuf]
+    uint32_t nqueue, ncand;    // (the same in every lane)
+};
+
+// The second stage for the last n <= 32 queued addresses, one per lane.
+template <int R, int KM, int ALPHA, bool SMEM>
+__device__ __forceinline__ void restore_second(const Geometry &G, const RestoreArgs &A, const RestoreConsts &C,
+                                               uint32_t dir, int szmax, WarpBufs &W, uint32_t n, uint32_t lane) {
+    __syncwarp();
+    W.nqueue -= n;
+    const uint2 v = lane < n ? W.queue[W.nqueue + lane] : make_uint2(0u, 0u);
+    const bool in = lane < n && rows_hot<KM == kAbove16 ? 2 : 3, R, KM, ALPHA, SMEM>(C, v.x, v.y);
+    const unsigned b = __ballot_sync(0xFFFFFFFFu, in);
+    if (in) W.cand[W.ncand + __popc(b & ((1u << lane) - 1u))] = v.x;
+    W.ncand += __popc(b);
+    __syncwarp();
+    if (W.ncand >= 32) flush_cands(G, A, dir, szmax, W.cand, W.hits, W.ncand, lane);
+}
+
+// The tests of two (c1, t) items per thread against the tile's c0 values.
+// Few pass the first stage, so a lane's survivor waits in the warp's queue
+// and the other rows are looked up 32 survivors at a time.  Bound by
+// instruction issue (68%).  Measured with the estimates that follow in the
+// same launch, against all rows at once and a launch of its own for the
+// estimates: core sketch, 18 M tests, 77,000 candidates 51 us (56 and the
+// gap); k = 18, 168 M tests 357 us (598 + 15).
+template <int R, int KM, int ALPHA, bool SMEM>
+__device__ __forceinline__ void restore_x2(const Geometry &G, const RestoreArgs &A, const RestoreConsts &C,
+                                           uint32_t dir, int szmax, const uint32_t *s_c0, uint32_t nc0, uint32_t c1a,
+                                           uint32_t ta, bool va, uint32_t c1b, uint32_t tb, bool vb, WarpBufs &W,
+                                           uint32_t lane) {
     const unsigned below = (1u << lane) - 1u;
     for (uint32_t q = 0; q < nc0; q++) {
         const uint32_t c0 = s_c0[q];  // same for the whole block
         uint32_t aa, ab;
-        const bool fa = va && restore_test<R, K16, ALPHA>(c0, c1a, k, kmask, lowbits, lowmask, A0, A0inv_k, hot2s, nw4,
-                                                           sh, aa);
-        const bool fb = vb && restore_test<R, K16, ALPHA>(c0, c1b, k, kmask, lowbits, lowmask, A0, A0inv_k, hot2s, nw4,
-                                                           sh, ab);
+        const bool fa = restore_first<R, KM, ALPHA, SMEM>(C, c0, c1a, ta, aa) && va;
+        const bool fb = restore_first<R, KM, ALPHA, SMEM>(C, c0, c1b, tb, ab) && vb;
         const unsigned ba = __ballot_sync(0xFFFFFFFFu, fa), bb = __ballot_sync(0xFFFFFFFFu, fb);
         if (!(ba | bb)) continue;
-        if (fa) cbuf[ccount + __popc(ba & below)] = aa;
-        ccount += __popc(ba);
-        if (fb) cbuf[ccount + __popc(bb & below)] = ab;
-        ccount += __popc(bb);
-        __syncwarp();
-        if (ccount >= 32) flush_cands(A, dir, cbuf, ccount, lane);
+        if (fa) W.queue[W.nqueue + __popc(ba & below)] = make_uint2(aa, c0);
+        W.nqueue += __popc(ba);
+        if (fb) W.queue[W.nqueue + __popc(bb & below)] = make_uint2(ab, c0);
+        W.nqueue += __popc(bb);
+        while (W.nqueue >= 32) restore_second<R, KM, ALPHA, SMEM>(G, A, C, dir, szmax, W, 32, lane);
     }
 }
 
-// Tiles t_begin, t_begin + t_step, ... below t_end of direction `dir`.
-__device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArgs &A, uint32_t dir, uint64_t t_begin,
-                                             uint64_t t_end, uint64_t t_step) {
-    extern __shared__ uint32_t smem[];
-    __shared__ uint32_t s_cbuf[8][kWarpBuf];
-    __shared__ uint32_t s_c0[kRestoreTileMax];
-    __shared__ bool s_stop;
-    __syncthreads();  // shared memory may still be in use by a previous call
-    // per-direction scalars picked with selects: indexing the parameter
-    // arrays with a run-time index would copy them to local memory
-    if (!(dir ? A.run[1] : A.run[0])) return;
-    const uint32_t n0 = dir ? A.n0[1] : A.n0[0];
-    const uint32_t n1 = dir ? A.n1[1] : A.n1[0];
-    if (n0 == 0 || n1 == 0) return;
-    const uint32_t k = G.k, kmask = (1u << k) - 1u;
-    const uint32_t hmask = (k >= 32u) ? 0u : ((1u << (32u - k)) - 1u);  // 32-k high bits
-    const uint32_t nw = (1u << k) >> 5;
-    const uint32_t A0 = dir ? G.h[1].A0 : G.h[0].A0;
-    const uint32_t A0inv = dir ? G.h[1].A0inv : G.h[0].A0inv;
-    const uint32_t *he0 = A.he + (uint64_t)dir * 2 * (1ull << k);
-    const uint32_t *he1 = he0 + (1ull << k);
-    const uint32_t *bm_dir = A.hotmap + (uint64_t)dir * G.r * nw;  // row i at bm_dir + i*nw
-    const uint64_t J = (uint64_t)n1 << A.ulog;
-    const uint32_t ntile0 = (n0 + A.tile0 - 1) / A.tile0;
-    const uint64_t nchunk = (J + A.jchunk - 1) / A.jchunk;
-    const uint64_t ntiles = (uint64_t)ntile0 * nchunk;
-    const uint64_t t_stop = t_end < ntiles ? t_end : ntiles;
-    if (t_begin >= t_stop) return;  // no tile of this direction for the block
+// One direction's restore job as a block needs it.
+struct RestoreDir {
+    uint32_t n0, n1, tile0;
+    int szmax;
+};
 
-    // rows 2..r-1 of the hot bitmap; row i is at hot2 + (i-2)*nw
-    const uint32_t *hot2 = bm_dir + 2 * nw;
-    if (A.smem_hot) {
-        uint32_t *sb = smem;
-        const uint32_t words = (G.r - 2) * nw;
-        for (uint32_t w = threadIdx.x; w < words; w += blockDim.x) sb[w] = hot2[w];
-        hot2 = sb;
-        __syncthreads();
-    }
+constexpr uint32_t kRestoreThreads = 256;
+constexpr uint32_t kRestoreItems = 2 * kRestoreThreads;  // (c1, t) items per tile
 
+__host__ __device__ __forceinline__ uint32_t restore_ulog(const Geometry &G) {
+    return G.k >= 16u ? 0u : 32u - 2u * G.k;
+}
+// c0 values per tile for `tests` tests in all: about tiles_per_block tiles
+// for each of (up to) 8 blocks per SM, so that the last wave is short
+__host__ __device__ __forceinline__ uint32_t restore_tile0(unsigned long long tests, uint32_t num_sms,
+                                                           uint32_t tiles_per_block) {
+    const unsigned long long per = tests / ((unsigned long long)num_sms * 8u * kRestoreThreads * tiles_per_block) + 1;
+    return (uint32_t)(per < kRestoreTileMax ? per : kRestoreTileMax);
+}
+__host__ __device__ __forceinline__ unsigned long long restore_tiles(const Geometry &G, uint32_t n0, uint32_t n1,
+                                                                     uint32_t tile0) {
+    if (!n0 || !n1) return 0;
+    const unsigned long long items = (unsigned long long)n1 << restore_ulog(G);
+    return (unsigned long long)((n0 + tile0 - 1) / tile0) * ((items + kRestoreItems - 1) / kRestoreItems);
+}
+
+// The tiles first, first + step, ... below stop of one direction (see
+// restore_body), by one way of testing.
+template <int R, int KM, int ALPHA, bool SMEM>
+__device__ __forceinline__ void restore_loop(const Geometry &G, const RestoreArgs &A, const RestoreConsts &C,
+                                             uint32_t dir, const RestoreDir &D, uint64_t first, uint64_t stop,
+                                             uint64_t step, WarpBufs &W, uint32_t *s_c0, bool *s_stop) {
     const uint32_t lane = threadIdx.x & 31u;
-    uint32_t *cbuf = s_cbuf[threadIdx.x >> 5];
-    uint32_t ccount = 0;  // warp-uniform
-    const uint32_t lowbits = (k >= 16u) ? (2u * k - 32u) : 0u;
-    const uint32_t lowmask = (1u << lowbits) - 1u;
-    const uint32_t iters = A.jchunk / blockDim.x;  // jchunk is a multiple of blockDim
-    // the specialised loop: k >= 16 (no enumeration of t), the hot bitmap in
-    // shared memory, at most 8 rows, an even number of c1 steps
-    const bool fast = k >= 16u && A.smem_hot && G.r <= 8u && (iters & 1u) == 0;
-    const uint32_t hot2s = (uint32_t)__cvta_generic_to_shared(smem);
-
-    for (uint64_t t = t_begin; t < t_stop; t += t_step) {
-        const uint32_t t0 = (uint32_t)(t / nchunk);
-        const uint64_t jc = t % nchunk;
-        const uint32_t c0_base = t0 * A.tile0;
-        const uint32_t nc0 = min(A.tile0, n0 - c0_base);
+    const uint32_t *he0 = A.he + (uint64_t)dir * 2 * (1ull << G.k);
+    const uint32_t *he1 = he0 + (1ull << G.k);
+    const uint64_t J = (uint64_t)D.n1 << C.ulog;
+    const uint64_t nchunk = (J + kRestoreItems - 1) / kRestoreItems;
+    // tile t covers c0 group t / nchunk and item chunk t % nchunk, stepped
+    // without dividing again
+    uint64_t t0 = first / nchunk, jc = first % nchunk;
+    const uint64_t t0_step = step / nchunk, jc_step = step % nchunk;
+    const uint32_t tm = (1u << C.ulog) - 1u;
+    for (uint64_t t = first; t < stop; t += step) {
+        const uint32_t c0_base = (uint32_t)t0 * D.tile0;
+        const uint32_t nc0 = min(D.tile0, D.n0 - c0_base);
+        // two (c1, t) items per thread
+        const uint64_t ja = jc * kRestoreItems + threadIdx.x, jb = ja + kRestoreThreads;
+        const bool va = ja < J, vb = jb < J;
+        const uint32_t c1a = va ? he1[ja >> C.ulog] : 0u, c1b = vb ? he1[jb >> C.ulog] : 0u;
         __syncthreads();
         // once K has passed its capacity the direction reports nothing but
         // the overload, so the rest of its enumeration is skipped (one read
         // of the shared counter per tile, the same decision for the block)
         if (threadIdx.x == 0)
-            s_stop = *reinterpret_cast<volatile unsigned long long *>(&A.stats->ncand[dir]) > A.cand_cap;
-        for (uint32_t q = threadIdx.x; q < nc0; q += blockDim.x) s_c0[q] = he0[c0_base + q];
+            *s_stop = *reinterpret_cast<volatile unsigned long long *>(&A.stats->ncand[dir]) > A.cand_cap;
+        for (uint32_t q = threadIdx.x; q < nc0; q += kRestoreThreads) s_c0[q] = he0[c0_base + q];
         __syncthreads();
-        if (s_stop) break;
-        if (fast) {
-            // two c1 values per thread and step (iters is even: jchunk = 2 blockDim)
-            for (uint32_t m = 0; m < iters; m += 2) {
-                const uint64_t ja = jc * A.jchunk + (uint64_t)m * blockDim.x + threadIdx.x;
-                const uint64_t jb = ja + blockDim.x;
-                const bool va = ja < J, vb = jb < J;
-                const uint32_t c1a = va ? he1[(uint32_t)ja] : 0u, c1b = vb ? he1[(uint32_t)jb] : 0u;
-                if (G.r == 4u && k == 16u && G.alpha == 8u) {  // the core-link sketch
-                    restore_c1x2<4, true, 8>(G, A, dir, s_c0, nc0, hot2s, nw, c1a, va, c1b, vb, A0, A0inv, cbuf,
-                                             ccount, lane);
-                    continue;
-                }
-                switch (G.r * 2u + (k == 16u ? 1u : 0u)) {
-#define SD_RESTORE_CASE(RR)                                                                                       \
-    case 2 * RR: restore_c1x2<RR, false, 0>(G, A, dir, s_c0, nc0, hot2s, nw, c1a, va, c1b, vb, A0, A0inv, cbuf,      \
-                                           ccount, lane); break;                                                  \
-    case 2 * RR + 1: restore_c1x2<RR, true, 0>(G, A, dir, s_c0, nc0, hot2s, nw, c1a, va, c1b, vb, A0, A0inv, cbuf,   \
-                                              ccount, lane); break;
-                    SD_RESTORE_CASE(3)
-                    SD_RESTORE_CASE(4)
-                    SD_RESTORE_CASE(5)
-                    SD_RESTORE_CASE(6)
-                    SD_RESTORE_CASE(7)
-                    SD_RESTORE_CASE(8)
-#undef SD_RESTORE_CASE
-                    default: break;
-                }
-            }
-            continue;
-        }
-        for (uint32_t m = 0; m < iters; m++) {
-            const uint64_t j = jc * A.jchunk + (uint64_t)m * blockDim.x + threadIdx.x;
-            const bool jvalid = j < J;
-            const uint32_t i1 = (uint32_t)(j >> A.ulog);
-            const uint32_t tt = (uint32_t)(j & ((1ull << A.ulog) - 1ull));
-            const uint32_t c1 = jvalid ? he1[i1] : 0u;
-            for (uint32_t q = 0; q < nc0; q++) {
-                const uint32_t c0 = s_c0[q];  // same for the whole block
-                const uint32_t L = c0 ^ c1;                 // BL(1): the low k bits of a
-                const uint32_t Q = A0 * L;
-                const uint32_t Qh = Q >> k, Ql = Q & kmask;
-                bool found = jvalid;
-                uint32_t u;
-                if (k >= 16u) {
-                    found = found && ((Ql >> (32u - k)) == (c0 & lowmask));
-                    u = c0 >> lowbits;
-                } else {
-                    u = (c0 << (32u - 2u * k)) | tt;
-                }
-                const uint32_t H = (A0inv * ((u - Qh) & hmask)) & hmask;
-                const uint32_t a = (H << k) | L;
-                for (uint32_t i = 2; i < G.r && found; i++)
-                    found = hot_at(hot2 + (uint64_t)(i - 2) * nw, dh_row(G, i, a, c0));
-                const unsigned fb = __ballot_sync(0xFFFFFFFFu, found);
-                if (!fb) continue;
-                // append the candidates to the warp's buffer; flush 32 at a time
-                if (found) cbuf[ccount + __popc(fb & ((1u << lane) - 1u))] = a;
-                ccount += __popc(fb);
-                __syncwarp();
-                if (ccount >= 32) flush_cands(A, dir, cbuf, ccount, lane);
-            }
+        if (*s_stop) break;
+        restore_x2<R, KM, ALPHA, SMEM>(G, A, C, dir, D.szmax, s_c0, nc0, c1a, (uint32_t)ja & tm, va, c1b,
+                                       (uint32_t)jb & tm, vb, W, lane);
+        t0 += t0_step;
+        jc += jc_step;
+        if (jc >= nchunk) {
+            jc -= nchunk;
+            t0++;
         }
     }
+    if (W.nqueue) restore_second<R, KM, ALPHA, SMEM>(G, A, C, dir, D.szmax, W, W.nqueue, lane);
     __syncwarp();
-    flush_cands(A, dir, cbuf, ccount, lane);
+    flush_cands(G, A, dir, D.szmax, W.cand, W.hits, W.ncand, lane);
 }
 
-// The tiles of direction 0 (tiles0 of them), then those of direction 1,
-// dealt round-robin to the blocks of a 1-D grid.
-__global__ void __launch_bounds__(256, 4)
-k_restore(Geometry G, RestoreArgs A, uint64_t tiles0) {
-    restore_body(G, A, 0, blockIdx.x, ~0ull, gridDim.x);
-    if (G.dirs > 1) {
+// Tiles t_begin, t_begin + t_step, ... below t_end of direction `dir`.
+// `stage`: rows 2.. of the hot bitmap are copied to shared memory first
+// (worth it for more than a few tests per thread), where they fit.
+template <int R>
+__device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArgs &A, uint32_t dir, RestoreDir D,
+                                             bool stage, uint64_t t_begin, uint64_t t_end, uint64_t t_step) {
+    extern __shared__ uint32_t smem[];
+    __shared__ unsigned long long s_hbuf[kRestoreThreads / 32][kWarpBuf];
+    __shared__ uint32_t s_cbuf[kRestoreThreads / 32][kWarpBuf];
+    __shared__ uint2 s_queue[kRestoreThreads / 32][96];
+    __shared__ uint32_t s_c0[kRestoreTileMax];
+    __shared__ bool s_stop;
+    __syncthreads();  // shared memory may still be in use by a previous call
+    const uint64_t ntiles = restore_tiles(G, D.n0, D.n1, D.tile0);
+    const uint64_t t_stop = t_end < ntiles ? t_end : ntiles;
+    if (t_begin >= t_stop) return;  // no tile of this direction for the block
+    RestoreConsts C;
+    C.k = G.k;
+    C.kmask = (1u << G.k) - 1u;
+    C.lowbits = G.k >= 16u ? 2u * G.k - 32u : 0u;
+    C.lowmask = (1u << C.lowbits) - 1u;
+    C.ulog = restore_ulog(G);
+    C.A0 = dir ? G.h[1].A0 : G.h[0].A0;
+    C.A0inv_k = (dir ? G.h[1].A0inv : G.h[0].A0inv) << G.k;
+    C.nw = (1u << G.k) >> 5;
+    C.alpha = G.alpha;
+    C.hot2 = A.hotmap + ((uint64_t)dir * G.r + 2u) * C.nw;
+    C.hot2s = (uint32_t)__cvta_generic_to_shared(smem);
+    if (stage) {
+        const uint32_t words = (G.r - 2) * C.nw;
+        if ((C.nw & 3u) == 0) {  // (rows of whole 16-byte words: k >= 7)
+            uint4 *to = reinterpret_cast<uint4 *>(smem);
+            const uint4 *from = reinterpret_cast<const uint4 *>(C.hot2);
+#pragma unroll 4
+            for (uint32_t w = threadIdx.x; w < words / 4; w += kRestoreThreads) to[w] = __ldcg(from + w);
+        } else {
+            for (uint32_t w = threadIdx.x; w < words; w += kRestoreThreads) smem[w] = __ldcg(C.hot2 + w);
+        }
+    }
+    const uint32_t wid = threadIdx.x >> 5;
+    WarpBufs W{s_queue[wid], s_cbuf[wid], s_hbuf[wid], 0u, 0u};
+#define SD_RESTORE(KM, ALPHA, SMEM) \
+    restore_loop<R, KM, ALPHA, SMEM>(G, A, C, dir, D, t_begin, t_stop, t_step, W, s_c0, &s_stop)
+    if (stage) {
+        if (R == 4 && G.k == 16u && G.alpha == 8u) SD_RESTORE(kIs16, 8, true);  // the core-link sketch
+        else if (G.k == 16u) SD_RESTORE(kIs16, 0, true);
+        else if (G.k < 16u) SD_RESTORE(kBelow16, 0, true);
+        else SD_RESTORE(kAbove16, 0, true);
+    } else {
+        if (G.k == 16u) SD_RESTORE(kIs16, 0, false);
+        else if (G.k < 16u) SD_RESTORE(kBelow16, 0, false);
+        else SD_RESTORE(kAbove16, 0, false);
+    }
+#undef SD_RESTORE
+}
+
+// Largest SZ that Eq. 4 may report, in float, from sum_ln = sum of
+// ln(ZR(i) / (g 2^k)): (g - g psi^r) e^(-theta/g) (Eq. 4 solved for SZ; xfac
+// is the exponential), raised by a hundredth, above the float's error (at most g r
+// 1e-7, 0.004 for g = 4096 and r = 8).  The host recomputes it in double and drops the
+// hits above its own, so the report does not depend on this rounding.
+__device__ __forceinline__ int szmax_bound(const Geometry &G, float sum_ln, float xfac) {
+    const float psi = -expm1f(sum_ln / (float)G.r);
+    float pr = psi;
+    for (uint32_t i = 1; i < G.r; i++) pr *= psi;
+    return (int)fmaxf(0.0f, ((float)G.g - (float)G.g * pr) * xfac + 0.01f);
+}
+
+// The restore of a close whose row statistics the host has not seen: the
+// directions that run (no saturated row, the work bound within pair_cap),
+// the tiles and the SZ bound are worked out by every block from the
+// StatBlock.  The tiles of direction 0, then those of direction 1, are dealt
+// round-robin to the blocks.
+template <int R>
+__global__ void __launch_bounds__(kRestoreThreads, 4)
+k_restore(const __grid_constant__ Geometry G, const __grid_constant__ RestoreArgs A, uint64_t pair_cap, float xfac,
+          uint32_t num_sms) {
+    __shared__ uint32_t s_n[2][2];
+    __shared__ int s_szmax[2];
+    if (threadIdx.x < 16) {  // eight lanes per direction, one row each
+        const uint32_t d = threadIdx.x >> 3, i = threadIdx.x & 7u;
+        const bool live = d < G.dirs && i < G.r;
+        const unsigned long long zr = live ? A.stats->zr[d][i] : 1ull;
+        uint32_t n0 = d < G.dirs ? A.stats->nhot[d][0] : 0u, n1 = d < G.dirs ? A.stats->nhot[d][1] : 0u;
+        float ln = live ? logf((float)zr / ((float)G.g * (float)(1u << G.k))) : 0.0f;
+        const bool sat = (__ballot_sync(0xFFFFu, zr == 0ull) >> (8u * d) & 0xFFu) != 0u;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) ln += __shfl_xor_sync(0xFFFFu, ln, o);
+        if (sat || ((uint64_t)n0 << (32u - G.k)) > pair_cap) n0 = n1 = 0;
+        if (i == 0) {
+            const int szmax = n0 && n1 ? szmax_bound(G, ln, xfac) : 0;
+            s_n[d][0] = n0;
+            s_n[d][1] = n1;
+            s_szmax[d] = szmax;
+            if (blockIdx.x == 0) A.stats->szmax_used[d] = szmax;
+        }
+    }
+    __syncthreads();
+    const uint32_t ulog = restore_ulog(G);
+    const unsigned long long tests = ((unsigned long long)s_n[0][0] * s_n[0][1] +
+                                      (unsigned long long)s_n[1][0] * s_n[1][1]) << ulog;
+    // staging the bitmap costs a block 3 to 4 us, a test looked up without it
+    // an L2 round trip per row: stage from two tests per thread on
+    const bool stage = A.smem_hot && tests > (unsigned long long)gridDim.x * kRestoreThreads * 2u;
+    const uint32_t tile0 = restore_tile0(tests, num_sms, 4);
+    uint64_t tiles0 = 0;
+    for (uint32_t d = 0; d < G.dirs; d++) {
+        const RestoreDir D{s_n[d][0], s_n[d][1], tile0, s_szmax[d]};
         const uint64_t first = ((uint64_t)blockIdx.x + gridDim.x - tiles0 % gridDim.x) % gridDim.x;
-        restore_body(G, A, 1, first, ~0ull, gridDim.x);
+        restore_body<R>(G, A, d, D, stage, first, ~0ull, gridDim.x);
+        tiles0 += restore_tiles(G, D.n0, D.n1, D.tile0);
     }
 }
 
-// k_estimate: SZ(a) = zero bits of ULE(a), the AND of a's r estimators, for
-// every candidate in K (one warp per candidate, lanes over the estimator's
-// words); keeps (a, SZ) when SZ <= szmax.  A direction whose K overflowed its
-// capacity is skipped (it reports nothing).
-// Candidates q_begin, q_begin + q_step, ... below q_end of direction `dir`,
-// one warp each.
-__device__ __forceinline__ void estimate_body(const Geometry &G, const RestoreArgs &A, uint32_t dir, uint64_t q_begin,
-                                              uint64_t q_end, uint64_t q_step) {
+// SZ and hits of a whole K in memory (the staged join's): warps take 32
+// candidates at a time.  A direction whose K overflowed its capacity is
+// skipped (it reports nothing).
+__global__ void __launch_bounds__(256)
+k_estimate(Geometry G, RestoreArgs A) {
     __shared__ unsigned long long s_hbuf[8][kWarpBuf];
+    const uint32_t dir = blockIdx.y;
     if (!(dir ? A.run[1] : A.run[0])) return;
     const unsigned long long nk = A.stats->ncand[dir];
     if (nk > A.cand_cap) return;
-    const int szmax = dir ? A.szmax[1] : A.szmax[0];
-    const uint32_t A0 = dir ? G.h[1].A0 : G.h[0].A0;
-    const uint32_t lane = threadIdx.x & 31u;
-    unsigned long long *hbuf = s_hbuf[threadIdx.x >> 5];
-    uint32_t hcount = 0;
-    const uint32_t *gdir = A.grid + (uint64_t)dir * G.dir_words;
-    const uint32_t *cand = A.cand + (uint64_t)dir * A.cand_cap;
-    const uint64_t q_stop = q_end < nk ? q_end : nk;
-    if (G.wpc >= 4) {
-        // lpc lanes per candidate, each ANDing 16-byte chunks of the r
-        // estimators; the warp's 32 / lpc candidates are q, q + q_step, ...
-        const uint32_t chunks = G.wpc >> 2;
-        const uint32_t lpc = chunks < 32u ? chunks : 32u;
-        const uint32_t cpw = 32u / lpc, sub = lane / lpc, sl = lane % lpc;
-        const uint32_t kmask = (1u << G.k) - 1u;
-        for (uint64_t q0 = q_begin; q0 < q_stop; q0 += (uint64_t)cpw * q_step) {
-            const uint64_t q = q0 + (uint64_t)sub * q_step;
-            const bool ok = q < q_stop;
-            const uint32_t x = ok ? cand[q] : 0u;
-            const uint32_t c0 = dh0(A0, G.k, x);
-            uint32_t ones = 0;
-            if (ok) {
-                for (uint32_t c = sl; c < chunks; c += lpc) {
-                    uint4 ule = make_uint4(~0u, ~0u, ~0u, ~0u);
-#pragma unroll
-                    for (uint32_t i = 0; i < 8; i++) {
-                        if (i >= G.r) break;
-                        const uint32_t ci = i == 0 ? c0 : ((shr_clamp(x, (i - 1u) * G.alpha) & kmask) ^ c0);
-                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(gdir + (uint64_t)i * G.row_words +
-                                                                              (uint64_t)ci * G.wpc) + c);
-                        ule.x &= v.x; ule.y &= v.y; ule.z &= v.z; ule.w &= v.w;
-                    }
-                    ones += __popc(ule.x) + __popc(ule.y) + __popc(ule.z) + __popc(ule.w);
-                }
-            }
-            for (uint32_t o = lpc >> 1; o > 0; o >>= 1) ones += __shfl_xor_sync(0xFFFFFFFFu, ones, o);
-            const bool hit = ok && sl == 0 && (int)(G.g - ones) <= szmax;
-            const unsigned hb = __ballot_sync(0xFFFFFFFFu, hit);
-            if (!hb) continue;
-            if (hit) hbuf[hcount + __popc(hb & ((1u << lane) - 1u))] = ((unsigned long long)x << 32) | (G.g - ones);
-            hcount += __popc(hb);
-            __syncwarp();
-            if (hcount >= 32) flush_hits(A, dir, hbuf, hcount, lane);
-        }
-        __syncwarp();
-        flush_hits(A, dir, hbuf, hcount, lane);
-        return;
-    }
-    for (uint64_t q = q_begin; q < q_stop; q += q_step) {
-        const uint32_t x = cand[q];
-        const uint32_t c0 = dh0(A0, G.k, x);
-        uint32_t ones = 0;
-        for (uint32_t w = lane; w < G.wpc; w += 32) {
-            uint32_t ule = 0xFFFFFFFFu;
-            for (uint32_t i = 0; i < G.r; i++) {
-                const uint32_t ci = (i == 0) ? c0 : dh_row(G, i, x, c0);
-                ule &= __ldg(gdir + (uint64_t)i * G.row_words + (uint64_t)ci * G.wpc + w);
-            }
-            ones += __popc(ule);
-        }
-        ones = warp_sum(ones);
-        const uint32_t SZ = G.g - ones;
-        if ((int)SZ <= szmax) {
-            if (lane == 0) hbuf[hcount] = ((unsigned long long)x << 32) | SZ;
-            hcount++;
-            __syncwarp();
-            if (hcount >= 32) flush_hits(A, dir, hbuf, hcount, lane);
-        }
-    }
-    __syncwarp();
-    flush_hits(A, dir, hbuf, hcount, lane);
-}
-
-__global__ void __launch_bounds__(256)
-k_estimate(Geometry G, RestoreArgs A) {
-    const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    estimate_body(G, A, blockIdx.y, (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), ~0ull, nwarps);
+    const uint32_t wid = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+    const uint64_t step = (uint64_t)gridDim.x * 8 * 32;
+    for (uint64_t q = ((uint64_t)blockIdx.x * 8 + wid) * 32; q < nk; q += step)
+        estimate_warp(G, A, dir, dir ? A.szmax[1] : A.szmax[0], A.cand + (uint64_t)dir * A.cand_cap + q,
+                      (uint32_t)(nk - q < 32 ? nk - q : 32), s_hbuf[wid], lane);
 }
 
 // ------------------------------------------------------------------- sort
@@ -542,6 +609,149 @@ k_sort_small(unsigned long long *hits, uint64_t hits_cap, StatBlock *st, uint2 r
     const uint32_t dir = blockIdx.x;
     if (!(dir ? run.y : run.x)) return;
     sort_small_body(hits, hits_cap, st, dir);
+}
+
+// The end of a queued close: each direction's hits ordered by address
+// straight into pinned host memory, and the StatBlock after them.
+//
+// A list of n hits is cut at addresses: nb = n / 256 ranges, each sorted by
+// one block.  Every block finds its two cuts by itself, as quantiles of the
+// same sample of 2 or 4 hits per range, and reads the whole list: it keeps the
+// hits of its range in shared memory and counts those below, which is where
+// its part of the order begins.  So no block waits for another and one
+// launch does it: 29,000 hits in 21 us and 2,400 in 12 us with cold caches,
+// where the one-block sort and the sample sort's four launches took 42 and
+// 23 us and a host round trip.  Within a block a hit's place is the number
+// of smaller addresses (addresses are distinct).  A range with more than
+// kRangeKeys hits, or a list of more than kFinishMax, sets big_sort: the
+// host sorts it by the longer way.
+constexpr uint32_t kFinishThreads = 1024;
+constexpr uint32_t kFinishLoads = 4;       // 16-byte loads in flight per thread
+constexpr uint32_t kFinishBlocks = 128;    // ranges at most
+constexpr uint32_t kRangeKeys = 2048;
+
+// number of u32 v[j] < x, j < n, v padded to a multiple of 4 with ~0
+__device__ __forceinline__ uint32_t count_below(const uint32_t *v, uint32_t n, uint32_t x) {
+    uint32_t c = 0;
+    const uint4 *v4 = reinterpret_cast<const uint4 *>(v);
+    for (uint32_t j = 0; j < (n + 3) / 4; j++) {
+        const uint4 q = v4[j];
+        c += (q.x < x) + (q.y < x) + (q.z < x) + (q.w < x);
+    }
+    return c;
+}
+
+__global__ void __launch_bounds__(kFinishThreads)
+k_close_finish(const unsigned long long *__restrict__ hits, uint64_t hits_cap, StatBlock *st,
+               unsigned long long *__restrict__ out, uint64_t out_cap, unsigned long long *__restrict__ spare,
+               StatBlock *st_out) {
+    __shared__ unsigned long long s_key[kRangeKeys];
+    __shared__ __align__(16) uint32_t s_ip[kRangeKeys + 4];
+    __shared__ uint32_t s_cut[2], s_n, s_below;
+    __shared__ bool s_last;
+    const uint32_t dir = blockIdx.y;
+    const unsigned long long nh = st->nhits[dir];
+    const bool fits = nh <= hits_cap && nh <= kFinishMax;
+    const uint32_t n = fits ? (uint32_t)nh : 0u;
+    uint32_t nb = (n + 255u) / 256u;
+    if (nb > kFinishBlocks) nb = kFinishBlocks;
+    // a list beyond the host's buffer is left in `spare` on the device
+    const bool spared = n > out_cap;
+    if ((!fits || spared) && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->big_sort[dir], fits ? 2u : 1u);
+    if (blockIdx.x < nb) {
+        const unsigned long long *h = hits + (uint64_t)dir * hits_cap;
+        if (threadIdx.x == 0) {
+            s_cut[0] = 0u;
+            s_cut[1] = ~0u;
+            s_n = 0;
+            s_below = 0;
+        }
+        if (nb > 1) {
+            // range b: addresses in [cut b, cut b + 1), cut j the (per j)-th
+            // smallest of per nb samples (a range of 256 hits on average may
+            // come out eight times as long, one of 512 four times)
+            const uint32_t per = n <= 32768u ? 2u : 4u, m = per * nb;
+            for (uint32_t i = threadIdx.x; i < ((m + 3u) & ~3u); i += kFinishThreads)
+                s_ip[i] = i < m ? (uint32_t)(h[(uint64_t)i * n / m] >> 32) : ~0u;
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < m; i += kFinishThreads) {
+                const uint32_t x = s_ip[i], rank = count_below(s_ip, m, x);
+                if (rank == per * blockIdx.x && blockIdx.x > 0) s_cut[0] = x;
+                if (rank == per * (blockIdx.x + 1)) s_cut[1] = x;
+            }
+        }
+        __syncthreads();
+        const uint32_t lo = s_cut[0], hi = s_cut[1];
+        const bool tail = blockIdx.x + 1 == nb;  // the last range has no upper cut
+        const uint32_t lane = threadIdx.x & 31u;
+        uint32_t below = 0;
+        // two hits per load (the lists start on 16 bytes and have room for an
+        // even number)
+        for (uint32_t i0 = 0; i0 < n; i0 += 2u * kFinishThreads * kFinishLoads) {
+            uint4 v[kFinishLoads];
+#pragma unroll
+            for (uint32_t u = 0; u < kFinishLoads; u++) {
+                const uint32_t i = i0 + 2u * (u * kFinishThreads + threadIdx.x);
+                v[u] = i < n ? __ldcg(reinterpret_cast<const uint4 *>(h + i)) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kFinishLoads; u++) {
+                const uint32_t i = i0 + 2u * (u * kFinishThreads + threadIdx.x);
+                const bool l0 = i < n, l1 = i + 1 < n;
+                const bool in0 = l0 && v[u].y >= lo && (tail || v[u].y < hi);
+                const bool in1 = l1 && v[u].w >= lo && (tail || v[u].w < hi);
+                below += (uint32_t)(l0 && v[u].y < lo) + (uint32_t)(l1 && v[u].w < lo);
+                if (in0 || in1) {
+                    uint32_t at = atomicAdd(&s_n, (uint32_t)in0 + (uint32_t)in1);
+                    if (in0 && at < kRangeKeys) s_key[at] = (unsigned long long)v[u].y << 32 | v[u].x;
+                    at += in0;
+                    if (in1 && at < kRangeKeys) s_key[at] = (unsigned long long)v[u].w << 32 | v[u].z;
+                }
+            }
+        }
+        below = warp_sum(below);
+        if (lane == 0 && below) atomicAdd(&s_below, below);
+        __syncthreads();
+        const uint32_t cnt = s_n, first = s_below;
+        if (cnt > kRangeKeys) {
+            if (threadIdx.x == 0) atomicOr(&st->big_sort[dir], 1u);
+        } else {
+            for (uint32_t i = threadIdx.x; i < ((cnt + 3u) & ~3u); i += kFinishThreads)
+                s_ip[i] = i < cnt ? (uint32_t)(s_key[i] >> 32) : ~0u;
+            __syncthreads();
+            unsigned long long key[kRangeKeys / kFinishThreads];
+            uint32_t at[kRangeKeys / kFinishThreads];
+#pragma unroll
+            for (uint32_t u = 0; u < kRangeKeys / kFinishThreads; u++) {
+                const uint32_t i = u * kFinishThreads + threadIdx.x;
+                key[u] = i < cnt ? s_key[i] : 0ull;
+                at[u] = i < cnt ? count_below(s_ip, cnt, (uint32_t)(key[u] >> 32)) : 0u;
+            }
+            __syncthreads();
+#pragma unroll
+            for (uint32_t u = 0; u < kRangeKeys / kFinishThreads; u++)
+                if (u * kFinishThreads + threadIdx.x < cnt) s_key[at[u]] = key[u];
+            __syncthreads();
+            unsigned long long *o = (spared ? spare + (uint64_t)dir * hits_cap : out + (uint64_t)dir * out_cap) + first;
+            for (uint32_t i = threadIdx.x; i < cnt; i += kFinishThreads) o[i] = s_key[i];
+        }
+    }
+    // the last block: the StatBlock to the host, and zero for the next window
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&st->finish_done, 1u) == gridDim.x * gridDim.y - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const volatile uint32_t *from = reinterpret_cast<const volatile uint32_t *>(st);
+    uint32_t *to = reinterpret_cast<uint32_t *>(st_out);
+    uint32_t *clr = reinterpret_cast<uint32_t *>(st);
+    for (uint32_t i = threadIdx.x; i < sizeof(StatBlock) / 4; i += kFinishThreads) {
+        to[i] = from[i];
+        clr[i] = 0;
+    }
 }
 
 // Sort every segment keys[j*kSortSmall, (j+1)*kSortSmall) of keys[0, n) in
@@ -857,83 +1067,20 @@ __device__ __forceinline__ uint32_t segment_of(const unsigned long long *base, u
 // Every block takes a contiguous run of the jobs' restore tiles (tile_base:
 // host-computed tile offsets per segment), so that blocks share the work of
 // the jobs in proportion to their tiles.
-__global__ void __launch_bounds__(256, 4)
+template <int R>
+__global__ void __launch_bounds__(kRestoreThreads, 4)
 k_restore_many(const CloseJob *__restrict__ J, const unsigned long long *__restrict__ tile_base, uint32_t count) {
     const uint64_t total = tile_base[2 * count];
     const uint64_t per = (total + gridDim.x - 1) / gridDim.x;
     uint64_t a = (uint64_t)blockIdx.x * per;
     const uint64_t b = a + per < total ? a + per : total;
     while (a < b) {
-        const uint32_t sg = segment_of(tile_base, 2 * count, a);
+        const uint32_t sg = segment_of(tile_base, 2 * count, a), d = sg & 1u;
         const uint64_t end = tile_base[sg + 1] < b ? tile_base[sg + 1] : b;
         const CloseJob &j = J[sg >> 1];
-        restore_body(j.G, j.A, sg & 1u, a - tile_base[sg], end - tile_base[sg], 1);
-        a = end;
-    }
-}
-
-// Candidate offsets per segment (0 for a direction that did not run or
-// whose K overflowed its capacity), for the flat estimate below: one block,
-// 1024 segments at a time, a block scan per batch of segments.
-__global__ void __launch_bounds__(1024)
-k_cand_base(const CloseJob *__restrict__ J, uint32_t count, unsigned long long *__restrict__ base) {
-    __shared__ unsigned long long s_warp[32];
-    __shared__ unsigned long long s_carry;
-    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
-    for (uint32_t s0 = 0; s0 < 2 * count; s0 += blockDim.x) {
-        const uint32_t sg = s0 + threadIdx.x;
-        unsigned long long c = 0;
-        if (sg < 2 * count) {
-            const CloseJob &j = J[sg >> 1];
-            const uint32_t d = sg & 1u;
-            if (d < j.G.dirs && (d ? j.A.run[1] : j.A.run[0])) {
-                const unsigned long long nk = j.A.stats->ncand[d];
-                if (nk <= j.A.cand_cap) c = nk;
-            }
-        }
-        unsigned long long incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if ((int)lane >= o) incl += v;
-        }
-        if (lane == 31) s_warp[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            unsigned long long x = lane < (blockDim.x >> 5) ? s_warp[lane] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long v = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if ((int)lane >= o) x += v;
-            }
-            s_warp[lane] = x;  // inclusive over warps
-        }
-        __syncthreads();
-        const unsigned long long carry = s_carry;
-        const unsigned long long excl = carry + incl - c + (wid ? s_warp[wid - 1] : 0);
-        if (sg < 2 * count) base[sg] = excl;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) s_carry = carry + s_warp[(blockDim.x >> 5) - 1];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) base[2 * count] = s_carry;
-}
-
-// Every warp takes a contiguous run of the jobs' candidates.
-__global__ void __launch_bounds__(256)
-k_estimate_many(const CloseJob *__restrict__ J, const unsigned long long *__restrict__ cand_base, uint32_t count) {
-    const uint64_t total = cand_base[2 * count];
-    const uint64_t nwarps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    const uint64_t per = (total + nwarps - 1) / nwarps;
-    uint64_t a = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
-    const uint64_t b = a + per < total ? a + per : total;
-    while (a < b) {
-        const uint32_t sg = segment_of(cand_base, 2 * count, a);
-        const uint64_t end = cand_base[sg + 1] < b ? cand_base[sg + 1] : b;
-        const CloseJob &j = J[sg >> 1];
-        estimate_body(j.G, j.A, sg & 1u, a - cand_base[sg], end - cand_base[sg], 1);
+        const RestoreDir D{j.A.n0[d], j.A.n1[d], j.A.tile0, j.A.szmax[d]};
+        restore_body<R>(j.G, j.A, d, D, j.A.smem_hot && (end - a) * D.tile0 > 2u, a - tile_base[sg],
+                        end - tile_base[sg], 1);
         a = end;
     }
 }
@@ -972,6 +1119,10 @@ __global__ void k_reset_many(const CloseJob *__restrict__ J, uint64_t n4) {
 }
 
 // ---------------------------------------------------------------- launchers
+// the hot bitmap rows that k_restore stages in shared memory
+constexpr size_t kRestoreHotMax = (size_t)200 * 1024;
+static size_t restore_hot_bytes(const Geometry &G) { return (size_t)(G.r - 2) * ((1u << G.k) >> 5) * 4; }
+
 static unsigned grid_for(uint64_t items, unsigned threads, int num_sms, unsigned per_sm) {
     uint64_t b = (items + threads - 1) / threads;
     const uint64_t cap = (uint64_t)num_sms * per_sm;
@@ -992,46 +1143,47 @@ cudaError_t launch_compact(const uint32_t *hotmap, const Geometry &G, uint32_t *
     return cudaGetLastError();
 }
 
-// Tile shape of k_restore for A's sizes: preimages per (c0, c1), (c1, t)
-// items per tile, and c0 values per tile -- enough work per tile to amortise
-// its set-up while still giving every resident block about one tile.
+// c0 values per tile of a batched restore (its own tests, a tile per block).
 void prepare_restore(const Geometry &G, RestoreArgs &A, int num_sms, uint32_t tiles_per_block) {
-    const unsigned threads = 256;
-    A.ulog = (G.k >= 16u) ? 0u : (32u - 2u * G.k);
-    A.jchunk = 2 * threads;  // two c1 values per thread and step
     uint64_t tests = 0;
     for (uint32_t d = 0; d < G.dirs; d++)
-        if (A.run[d]) tests += (uint64_t)A.n0[d] * ((uint64_t)A.n1[d] << A.ulog);
-    // c0 values per tile: about tiles_per_block tiles for each of the
-    // (up to) 8 blocks per SM, so that the last wave of tiles is short
-    const uint64_t per_block = tests / ((uint64_t)num_sms * 8 * threads * tiles_per_block) + 1;
-    A.tile0 = (uint32_t)(per_block < kRestoreTileMax ? per_block : kRestoreTileMax);
-    const size_t hot_bytes = (size_t)(G.r - 2) * ((1u << G.k) >> 5) * 4;
-    A.smem_hot = hot_bytes <= (size_t)200 * 1024;
+        if (A.run[d]) tests += (uint64_t)A.n0[d] * ((uint64_t)A.n1[d] << restore_ulog(G));
+    A.tile0 = restore_tile0(tests, (uint32_t)num_sms, tiles_per_block);
+    A.smem_hot = restore_hot_bytes(G) <= kRestoreHotMax;
 }
 
 // k_restore tiles of direction d (the same count the kernel derives)
 static uint64_t restore_tiles_dir(const Geometry &G, const RestoreArgs &A, uint32_t d) {
-    if (d >= G.dirs || !A.run[d] || A.n0[d] == 0 || A.n1[d] == 0) return 0;
-    const uint64_t t0 = (A.n0[d] + A.tile0 - 1) / A.tile0;
-    const uint64_t nc = (((uint64_t)A.n1[d] << A.ulog) + A.jchunk - 1) / A.jchunk;
-    return t0 * nc;
+    return d < G.dirs && A.run[d] ? restore_tiles(G, A.n0[d], A.n1[d], A.tile0) : 0;
 }
 
-cudaError_t launch_restore(const Geometry &G, RestoreArgs A, int num_sms, cudaStream_t s) {
-    const unsigned threads = 256;
-    prepare_restore(G, A, num_sms, 4);
-    const size_t hot_bytes = (size_t)(G.r - 2) * ((1u << G.k) >> 5) * 4;
-    const size_t smem = A.smem_hot ? hot_bytes : 16;
-    const uint64_t tiles0 = restore_tiles_dir(G, A, 0);
-    const uint64_t total = tiles0 + restore_tiles_dir(G, A, 1);
-    if (total == 0) return cudaSuccess;
+template <typename F3, typename F4, typename F5, typename F6, typename F7, typename F8>
+static const void *by_rows(uint32_t r, F3 f3, F4 f4, F5 f5, F6 f6, F7 f7, F8 f8) {
+    const void *f[] = {(const void *)f3, (const void *)f4, (const void *)f5, (const void *)f6, (const void *)f7,
+                       (const void *)f8};
+    return r >= 3 && r <= 8 ? f[r - 3] : nullptr;
+}
+
+cudaError_t launch_restore(const Geometry &G, RestoreArgs A, uint64_t pair_cap, float xfac, int num_sms,
+                           cudaStream_t s) {
+    const void *kern = by_rows(G.r, k_restore<3>, k_restore<4>, k_restore<5>, k_restore<6>, k_restore<7>,
+                               k_restore<8>);
+    if (!kern) return cudaErrorInvalidValue;
+    A.smem_hot = restore_hot_bytes(G) <= kRestoreHotMax;
+    const size_t smem = A.smem_hot ? restore_hot_bytes(G) : 16;
     int per_sm = 0;
-    cudaError_t e = prepare_launch(reinterpret_cast<const void *>(k_restore), (int)threads, smem, &per_sm);
+    cudaError_t e = prepare_launch(kern, (int)kRestoreThreads, smem, &per_sm);
     if (e != cudaSuccess) return e;
-    uint64_t blocks = (uint64_t)num_sms * per_sm;
-    if (total < blocks) blocks = total;
-    k_restore<<<(unsigned)blocks, threads, smem, s>>>(G, A, tiles0);
+    uint32_t sms = (uint32_t)num_sms;
+    void *args[] = {const_cast<Geometry *>(&G), &A, &pair_cap, &xfac, &sms};
+    return cudaLaunchKernel(kern, dim3((unsigned)(num_sms * per_sm)), dim3(kRestoreThreads), args, smem, s);
+}
+
+cudaError_t launch_close_finish(const unsigned long long *hits, uint64_t hits_cap, StatBlock *st,
+                                unsigned long long *out, uint64_t out_cap, unsigned long long *spare,
+                                StatBlock *st_out, uint32_t dirs, cudaStream_t s) {
+    k_close_finish<<<dim3(kFinishBlocks, dirs), kFinishThreads, 0, s>>>(hits, hits_cap, st, out, out_cap, spare,
+                                                                        st_out);
     return cudaGetLastError();
 }
 
@@ -1124,13 +1276,10 @@ cudaError_t launch_stats_many(const CloseJob *J, uint32_t count, const Geometry 
 }
 
 cudaError_t launch_restore_many(const CloseJob *J, const CloseJob *Jh, uint32_t count, unsigned long long *tile_base_d,
-                                unsigned long long *tile_base_h, unsigned long long *cand_base_d, int num_sms,
-                                cudaStream_t s, int *launches) {
+                                unsigned long long *tile_base_h, int num_sms, cudaStream_t s, int *launches) {
     *launches = 0;
     const Geometry &G = Jh[0].G;
-    const unsigned threads = 256;
-    const size_t hot_bytes = (size_t)(G.r - 2) * ((1u << G.k) >> 5) * 4;
-    const size_t smem = Jh[0].A.smem_hot ? hot_bytes : 16;
+    const size_t smem = Jh[0].A.smem_hot ? restore_hot_bytes(G) : 16;
     unsigned long long acc = 0;
     bool any = false;
     for (uint32_t i = 0; i < count; i++) {
@@ -1146,23 +1295,24 @@ cudaError_t launch_restore_many(const CloseJob *J, const CloseJob *Jh, uint32_t 
                                     cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     if (acc > 0) {
+        const void *kern = by_rows(G.r, k_restore_many<3>, k_restore_many<4>, k_restore_many<5>, k_restore_many<6>,
+                                   k_restore_many<7>, k_restore_many<8>);
+        if (!kern) return cudaErrorInvalidValue;
         int per_sm = 0;
-        e = prepare_launch(reinterpret_cast<const void *>(k_restore_many), (int)threads, smem, &per_sm);
+        e = prepare_launch(kern, (int)kRestoreThreads, smem, &per_sm);
         if (e != cudaSuccess) return e;
         const uint64_t blocks = std::min<uint64_t>((uint64_t)num_sms * per_sm, acc);
-        k_restore_many<<<(unsigned)blocks, threads, smem, s>>>(J, tile_base_d, count);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        void *args[] = {&J, &tile_base_d, &count};
+        e = cudaLaunchKernel(kern, dim3((unsigned)blocks), dim3(kRestoreThreads), args, smem, s);
+        if (e != cudaSuccess) return e;
         ++*launches;
     }
-    k_cand_base<<<1, 1024, 0, s>>>(J, count, cand_base_d);
-    k_estimate_many<<<(unsigned)num_sms * 8, 256, 0, s>>>(J, cand_base_d, count);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int ssmem = kSortSmall * (int)sizeof(unsigned long long);
     int per_sm = 0;
     e = prepare_launch(reinterpret_cast<const void *>(k_sort_small_many), 1024, ssmem, &per_sm);
     if (e != cudaSuccess) return e;
     k_sort_small_many<<<dim3(G.dirs, count), 1024, ssmem, s>>>(J);
-    *launches += 3;
+    *launches += 1;
     return cudaGetLastError();
 }
 

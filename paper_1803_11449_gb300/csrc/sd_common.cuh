@@ -113,10 +113,12 @@ struct StatBlock {
     unsigned long long ncand[2];
     unsigned long long nhits[2];
     unsigned int nhot[2][kMaxRows];
-    unsigned int big_sort[2];  // 1: hits did not fit the one-block sort
-    unsigned int pad[2];
+    unsigned int big_sort[2];  // 1: hits did not fit the one-launch sort; 2: ordered, but on the device
+    int szmax_used[2];         // k_restore's SZ bound
     unsigned long long jcount[2][kMaxRows];  // staged join: entries stage i produced
     unsigned int rows_done[2][2];  // k_plane_scan: tiles of rows 0 and 1 counted
+    unsigned int finish_done;      // k_close_finish: blocks done
+    unsigned int pad;
 };
 
 struct RestoreArgs {
@@ -130,10 +132,8 @@ struct RestoreArgs {
     uint32_t n0[2], n1[2];
     int32_t szmax[2];        // largest reported SZ; -1: none
     uint32_t run[2];
-    uint32_t ulog;           // log2 of the preimage count per (c0, c1): max(0, 32-2k)
-    uint32_t tile0;          // c0 values per block tile
-    uint32_t jchunk;         // (c1, t) items per block tile
-    int smem_hot;            // rows 2..r-1 of the hot bitmap staged in shared memory
+    uint32_t tile0;          // c0 values per block tile (batched closes)
+    int smem_hot;            // rows 2..r-1 of the hot bitmap fit shared memory
 };
 
 // One window close of a batch (sd_close_many over handles of one DHLA
@@ -227,7 +227,17 @@ cudaError_t launch_row_stats(const uint32_t *grid, const Geometry &G, int zhot, 
                              StatBlock *st, int num_sms, cudaStream_t s);
 // HE(i) for rows 0..rows-1 of every direction, ascending: he[dir][row][2^k]
 cudaError_t launch_compact(const uint32_t *hotmap, const Geometry &G, uint32_t *he, uint32_t rows, cudaStream_t s);
-cudaError_t launch_restore(const Geometry &G, RestoreArgs A, int num_sms, cudaStream_t s);
+// K, SZ and hits of a close whose statistics the host has not seen (see
+// k_restore); xfac = e^(-theta/g)
+cudaError_t launch_restore(const Geometry &G, RestoreArgs A, uint64_t pair_cap, float xfac, int num_sms,
+                           cudaStream_t s);
+// hits a queued close orders by itself, per direction: into the host's `out`
+// (out_cap keys per direction) or, for more than that, `spare` (as large as
+// the hit lists; big_sort 2); longer lists set big_sort 1
+constexpr uint32_t kFinishMax = 1u << 16;
+cudaError_t launch_close_finish(const unsigned long long *hits, uint64_t hits_cap, StatBlock *st,
+                                unsigned long long *out, uint64_t out_cap, unsigned long long *spare,
+                                StatBlock *st_out, uint32_t dirs, cudaStream_t s);
 cudaError_t launch_estimate(const Geometry &G, const RestoreArgs &A, int num_sms, cudaStream_t s);
 // Host: DHLA layout and hash constants for a valid *p (as sd_create sets them).
 void geometry_of(const sd_params *p, Geometry *out);
@@ -239,11 +249,10 @@ void geometry_of(const sd_params *p, Geometry *out);
 // [kSortSmall]; the reset of every job's counters and (stats_done < 2) DHLA.
 cudaError_t launch_stats_many(const CloseJob *J, uint32_t count, const Geometry &G, int num_sms, cudaStream_t s);
 void prepare_restore(const Geometry &G, RestoreArgs &A, int num_sms, uint32_t tiles_per_block);
-// (restore and estimate spread all jobs' tiles / candidates over the whole
-// grid: tile_base_* and cand_base_d hold 2 count + 1 offsets)
+// (the restore spreads all jobs' tiles over the whole grid: tile_base_* hold
+// 2 count + 1 offsets)
 cudaError_t launch_restore_many(const CloseJob *J, const CloseJob *Jh, uint32_t count, unsigned long long *tile_base_d,
-                                unsigned long long *tile_base_h, unsigned long long *cand_base_d, int num_sms,
-                                cudaStream_t s, int *launches);
+                                unsigned long long *tile_base_h, int num_sms, cudaStream_t s, int *launches);
 cudaError_t launch_gather_many(const CloseJob *J, uint32_t count, StatBlock *st_out, unsigned long long *hits_out,
                                cudaStream_t s);
 cudaError_t launch_reset_many(const CloseJob *J, uint32_t count, const Geometry &G, int num_sms, cudaStream_t s);
