@@ -54,7 +54,7 @@ constexpr uint32_t kPlaneThreads = 512;   // k_plane_bin / k_plane_count block
 constexpr uint32_t kApplyThreads = 512;   // k_plane_apply block (1024 where one plane fills the block's shared memory)
 constexpr uint32_t kHeldReservations = 2;  // reservation results a thread holds across the scatter
 constexpr uint32_t kBinTilesPerBlock = 8;   // k_plane_bin tiles per block (blocks retire as a round runs)
-constexpr uint32_t kApplyUnitsPerBlock = 4; // k_plane_apply units per block
+constexpr uint32_t kApplyUnitsPerBlock = 4; // k_plane_apply units per block, at most
 
 __device__ __forceinline__ uint32_t h1v(uint64_t A1, uint64_t B1, uint32_t lg, uint32_t y) {
     return (uint32_t)((A1 * (uint64_t)y + B1) >> (64u - lg));
@@ -253,7 +253,8 @@ __device__ __forceinline__ void bin_hash(uint32_t cnt, const uint32_t (&ps)[PPT]
 
 template <int DIRS, int PPT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
-k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArgs P) {
+k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArgs P, uint32_t head,
+            uint32_t tile) {
     constexpr int E = PPT * DIRS;
     extern __shared__ unsigned long long sm64[];
     __shared__ uint32_t s_warp[32];
@@ -266,7 +267,7 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
     uint32_t *hist = reinterpret_cast<uint32_t *>(dst + NB);       // [NB] entries of each plane in the tile
     uint32_t *offs = hist + NB;                                    // [NB] first sorted position of each plane
     const uint64_t A1a = G.h[0].A1, B1a = G.h[0].B1, A1b = G.h[1].A1, B1b = G.h[1].B1;
-    const uint64_t ntiles = (n + TP - 1) / TP;
+    const uint64_t ntiles = (n + tile - 1) / tile;  // (tile <= TP pairs each)
     const bool vec = ((uintptr_t)pairs & 15u) == 0;
     // planes owned by this thread in the scan (contiguous chunk)
     const uint32_t per = (NB + blockDim.x - 1) / blockDim.x;
@@ -274,9 +275,9 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
     // this thread's pairs of tile t: 2-pair units threadIdx.x + j blockDim.x
     // (coalesced 16-byte loads where the buffer allows)
     auto load_tile = [&](uint64_t t, uint32_t (&ps)[PPT], uint32_t (&pt)[PPT]) {
-        const uint64_t base = t * TP;
+        const uint64_t base = t * tile;
         const uint64_t left = t < ntiles ? n - base : 0;
-        const uint32_t cnt = left < TP ? (uint32_t)left : TP;
+        const uint32_t cnt = left < tile ? (uint32_t)left : tile;
 #pragma unroll
         for (int j = 0; j < PPT / 2; j++) {
             const uint32_t pu = threadIdx.x + (uint32_t)j * blockDim.x;
@@ -296,12 +297,17 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
         }
     };
     for (uint32_t b = threadIdx.x; b < NB; b += blockDim.x) hist[b] = 0;
+    if (head && blockIdx.x == 0 && threadIdx.x == 0) {  // the pair before `pairs`
+        const uint32_t s = pairs[-2], t = pairs[-1];
+        set_key_bits<DIRS>(G, P, h1v(A1a, B1a, lg, t), s);
+        if (DIRS == 2) set_key_bits<DIRS>(G, P, g + h1v(A1b, B1b, lg, s), t);
+    }
     __syncthreads();
     uint32_t nps[PPT], npt[PPT];  // the next tile's pairs, loaded while the current one is written out
     load_tile(blockIdx.x, nps, npt);
     for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const uint64_t left = n - t * TP;
-        const uint32_t cnt = left < TP ? (uint32_t)left : TP;
+        const uint64_t left = n - t * tile;
+        const uint32_t cnt = left < tile ? (uint32_t)left : tile;
         const bool full = cnt == TP;
         uint32_t key[E], tag[E];
         if (full) bin_hash<DIRS, PPT, true>(cnt, nps, npt, g, lg, A1a, B1a, A1b, B1b, hist, key, tag);
@@ -404,7 +410,6 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
                [&](uint32_t i, uint32_t v) { P.unit_start[i] = v; }, s_warp);
     if (threadIdx.x == 0) {
         P.ctl[0] = 0;
-        P.ctl[1] = 0;
         P.ctl[2] = 0;
     }
 }
@@ -431,36 +436,42 @@ template <int R, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
     extern __shared__ uint4 pl4_all[];  // nbuf planes of ps words
-    __shared__ uint32_t s_unit;
+    __shared__ uint4 s_unit[kApplyUnitsPerBlock];  // (plane, first entry, entries, -) of the block's units
     __shared__ uint32_t s_warp[32];
     __shared__ bool s_last;
     const uint32_t NB = P.nbins;
     const uint32_t rw = (1u << G.k) >> 5;
+    // a block takes per_block consecutive units (the grid holds enough
+    // blocks for every unit), so that blocks retire as the round
+    // proceeds and other streams' work (a window close) gets SMs in between.
+    // Their planes are found at once: every thread looks at its planes'
+    // ranges of units, one L2 round trip instead of a search of ten for each
+    // unit (2^26 pairs of the core sketch: 270 us, 280 with searches and a
+    // shared unit counter; 128 KiB planes, one block per SM: 345 and 362).
+    const uint32_t x0 = blockIdx.x * per_block;
     const uint32_t total = P.unit_start[NB];
-    // a block takes at most per_block units (the grid holds enough blocks
-    // for every unit), so that blocks retire as the round proceeds and
-    // other streams' work (a window close) gets SMs in between
-    for (uint32_t it = 0; it < per_block; it++) {
+    for (uint32_t b = threadIdx.x; b < NB; b += THREADS) {
+        const uint32_t u0 = P.unit_start[b], u1 = P.unit_start[b + 1];
+        if (u1 <= x0 || u0 >= x0 + per_block) continue;
+        const uint32_t off = P.binoff[b], n = min(P.cnt[b], P.cap[b]);
+#pragma unroll
+        for (uint32_t j = 0; j < kApplyUnitsPerBlock; j++) {
+            const uint32_t x = x0 + j;
+            if (j >= per_block || x < u0 || x >= u1) continue;
+            const uint32_t at = (x - u0) * P.unit;
+            s_unit[j] = make_uint4(b, off + at, n - at < P.unit ? n - at : P.unit, 0u);
+        }
+    }
+    for (uint32_t it = 0; it < per_block && x0 + it < total; it++) {
         uint4 *pl4 = pl4_all + (size_t)(it % nbuf) * (P.ps / 4);
         uint32_t *pl = reinterpret_cast<uint32_t *>(pl4);
         if (threadIdx.x == 0) {
             if (nbuf == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
             else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            s_unit = atomicAdd(&P.ctl[1], 1u);
         }
-        __syncthreads();  // this buffer is free again; the unit is known
-        const uint32_t x = s_unit;
-        if (x >= total) break;
-        uint32_t lo = 0, hi = NB;  // the plane b with unit_start[b] <= x < unit_start[b + 1]
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (P.unit_start[mid] <= x) lo = mid;
-            else hi = mid;
-        }
-        const uint32_t b = lo;
-        const uint32_t beg = P.binoff[b] + (x - P.unit_start[b]) * P.unit;
-        const uint32_t stop = P.binoff[b] + min(P.cnt[b], P.cap[b]);
-        const uint32_t end = stop - beg < P.unit ? stop : beg + P.unit;
+        __syncthreads();  // this buffer is free again; the units are known
+        const uint4 unit = s_unit[it];
+        const uint32_t b = unit.x, beg = unit.y, end = beg + unit.z;
         const uint32_t A0 = (b >> G.lg) ? G.h[1].A0 : G.h[0].A0;
         for (uint32_t i = threadIdx.x; i < P.ps / 4; i += blockDim.x) pl4[i] = make_uint4(0, 0, 0, 0);
         __syncthreads();
@@ -495,7 +506,9 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
     }
-    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    // (shared memory must outlive the reductions' reads; the reductions
+    // themselves are complete when the kernel is)
+    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     // the last block: the next round's bins from this round's counts
     if (!last_block(&P.ctl[2], &s_last)) return;
     write_layout(P, true, s_warp);
@@ -548,7 +561,7 @@ size_t plane_bin_smem_bytes(uint32_t tile_pairs, uint32_t dirs, uint32_t nbins) 
 
 template <int DIRS, int PPT, int THREADS>
 static cudaError_t launch_plane_bin(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P,
-                                    int num_sms, cudaStream_t s) {
+                                    uint32_t head, int num_sms, cudaStream_t s) {
     auto kern = k_plane_bin<DIRS, PPT, THREADS>;
     const size_t smem = plane_bin_smem_bytes(P.tile_pairs, DIRS, P.nbins);
     int per_sm = 0;
@@ -556,12 +569,22 @@ static cudaError_t launch_plane_bin(const uint32_t *pairs, uint64_t n, const Geo
     if (e != cudaSuccess) return e;
     // about kBinTilesPerBlock tiles per block (not one persistent block per
     // SM), so that blocks retire as the round proceeds and other streams'
-    // work gets SMs in between
-    const uint64_t tiles = (n + P.tile_pairs - 1) / P.tile_pairs;
+    // work gets SMs in between.  A round of few waves of tiles is cut into as
+    // many equal ones instead, so that the last wave is not half empty
+    // (4,000,000 pairs are 3.2 waves of full tiles: 34 us, 35 with those).
+    const uint64_t resident = (uint64_t)num_sms * per_sm;
+    uint32_t tile = P.tile_pairs;
+    uint64_t tiles = (n + tile - 1) / tile;
     uint64_t blocks = (tiles + kBinTilesPerBlock - 1) / kBinTilesPerBlock;
-    if (blocks < (uint64_t)num_sms * per_sm) blocks = (uint64_t)num_sms * per_sm;
+    if (blocks < resident) {
+        const uint64_t waves = (tiles + resident - 1) / resident;
+        const uint64_t even = (n + waves * resident - 1) / (waves * resident);
+        if (even + 1 < tile) tile = (uint32_t)((even + 1) & ~1ull);
+        tiles = (n + tile - 1) / tile;
+        blocks = resident;
+    }
     if (tiles < blocks) blocks = tiles;
-    kern<<<(unsigned)blocks, THREADS, smem, s>>>(pairs, n, G, P);
+    kern<<<(unsigned)blocks, THREADS, smem, s>>>(pairs, n, G, P, head, tile);
     return cudaGetLastError();
 }
 
@@ -569,12 +592,12 @@ static cudaError_t launch_plane_bin(const uint32_t *pairs, uint64_t n, const Geo
 // 8192: 1024 threads with 8 each (one block per SM)
 template <int DIRS>
 static cudaError_t launch_plane_bin_d(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P,
-                                      int num_sms, cudaStream_t s) {
+                                      uint32_t head, int num_sms, cudaStream_t s) {
     switch (P.tile_pairs) {
-        case 1024: return launch_plane_bin<DIRS, 2, 512>(pairs, n, G, P, num_sms, s);
-        case 2048: return launch_plane_bin<DIRS, 4, 512>(pairs, n, G, P, num_sms, s);
-        case 4096: return launch_plane_bin<DIRS, 8, 512>(pairs, n, G, P, num_sms, s);
-        case 8192: return launch_plane_bin<DIRS, 8, 1024>(pairs, n, G, P, num_sms, s);
+        case 1024: return launch_plane_bin<DIRS, 2, 512>(pairs, n, G, P, head, num_sms, s);
+        case 2048: return launch_plane_bin<DIRS, 4, 512>(pairs, n, G, P, head, num_sms, s);
+        case 4096: return launch_plane_bin<DIRS, 8, 512>(pairs, n, G, P, head, num_sms, s);
+        case 8192: return launch_plane_bin<DIRS, 8, 1024>(pairs, n, G, P, head, num_sms, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -582,27 +605,38 @@ static cudaError_t launch_plane_bin_d(const uint32_t *pairs, uint64_t n, const G
 template <int R>
 static cudaError_t launch_plane_apply(const Geometry &G, const PlaneArgs &P, uint64_t n, int num_sms,
                                      cudaStream_t s) {
-    const uint32_t nbuf = (size_t)P.ps * 8 <= (size_t)100 * 1024 ? 2u : 1u;
-    auto kern = nbuf == 2 ? k_plane_apply<R, kApplyThreads> : k_plane_apply<R, 2 * kApplyThreads>;
-    const uint32_t threads = nbuf == 2 ? kApplyThreads : 2 * kApplyThreads;
-    const size_t smem = (size_t)P.ps * 4 * nbuf;
+    // two plane buffers of 512 threads where they fit; one plane of 1024
+    // threads per block beyond that
+    const bool two = (size_t)P.ps * 8 <= (size_t)100 * 1024;
+    auto kern = two ? k_plane_apply<R, kApplyThreads> : k_plane_apply<R, 2 * kApplyThreads>;
+    const uint32_t threads = two ? kApplyThreads : 2 * kApplyThreads;
+    const size_t plane = (size_t)P.ps * 4;
     int per_sm = 0;
-    cudaError_t e = prepare_launch(reinterpret_cast<const void *>(kern), (int)threads, smem, &per_sm);
+    cudaError_t e = prepare_launch(reinterpret_cast<const void *>(kern), (int)threads, two ? 2 * plane : plane, &per_sm);
     if (e != cudaSuccess) return e;
     // units of the round: at most (keys + slack) / unit + one partial unit per plane
     const uint64_t keys = (uint64_t)(P.nbins / G.g) * n;
     const uint64_t most = (keys + keys / 8 + 40ull * P.nbins) / P.unit + P.nbins;
-    const uint32_t per_block = kApplyUnitsPerBlock;
-    uint64_t blocks = (most + per_block - 1) / per_block;
-    if (blocks < (uint64_t)num_sms * per_sm) blocks = (uint64_t)num_sms * per_sm;
+    // kApplyUnitsPerBlock of them per block, fewer in a round too short for
+    // two waves of such blocks; a block of one unit needs one buffer
+    const uint64_t waves = most / ((uint64_t)num_sms * per_sm * 2);
+    const uint64_t per_block = waves < 1 ? 1 : (waves < kApplyUnitsPerBlock ? waves : kApplyUnitsPerBlock);
+    const uint32_t nbuf = two && per_block > 1 ? 2u : 1u;
+    const uint64_t blocks = (most + per_block - 1) / per_block;
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    kern<<<(unsigned)blocks, threads, smem, s>>>(G, P, nbuf, per_block);
+    kern<<<(unsigned)blocks, threads, plane * nbuf, s>>>(G, P, nbuf, (uint32_t)per_block);
     return cudaGetLastError();
 }
 
 cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
                                cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs) {
     if (n == 0) return cudaSuccess;
+    // pairs that start 8 bytes past a 16-byte boundary: the first one is set
+    // directly, the rest is read in 16-byte loads (4,000,000 of them: bin 35
+    // us where 4-byte loads took 40)
+    const uint32_t head = ((uintptr_t)pairs & 15u) == 8 && n > 1 ? 1u : 0u;
+    pairs += 2 * head;
+    n -= head;
     if (layout == kLayoutScale) {
         if (prev_pairs == 0) return cudaErrorInvalidValue;
         k_plane_layout<<<1, 1024, 0, s>>>(P, n, prev_pairs);
@@ -620,8 +654,8 @@ cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry
         kern<<<(unsigned)blocks, kPlaneThreads, smem, s>>>(pairs, n, G, P);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    cudaError_t e = G.dirs == 2 ? launch_plane_bin_d<2>(pairs, n, G, P, num_sms, s)
-                                : launch_plane_bin_d<1>(pairs, n, G, P, num_sms, s);
+    cudaError_t e = G.dirs == 2 ? launch_plane_bin_d<2>(pairs, n, G, P, head, num_sms, s)
+                                : launch_plane_bin_d<1>(pairs, n, G, P, head, num_sms, s);
     if (e != cudaSuccess) return e;
     switch (G.r) {
         case 3: return launch_plane_apply<3>(G, P, n, num_sms, s);
