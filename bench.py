@@ -741,10 +741,9 @@ def run_shard(args, rank, world, local):
 
 
 def run_noalloc(args, rank, world, local):
-    """sd_update_noalloc (the binned update with its scratch in a fixed
-    array inside the library) on the core window, beside sd_update in the
-    same binned mode (5) and in the default mode: CUDA events around each
-    call, pairs resident in HBM (one JSON line)."""
+    """sd_update_noalloc (set in place, no scratch) on the core window, beside
+    sd_update binned by slice (mode 5) and in the default mode: CUDA events
+    around each call, pairs resident in HBM (one JSON line)."""
     import torch
 
     from paper_1803_11449_gb300 import build as b

@@ -179,7 +179,7 @@ k_update(const uint32_t *__restrict__ pairs, uint64_t n, uint32_t *__restrict__ 
 }
 
 // Pairs that are only 4-byte aligned (an odd word offset): one pair per
-// thread with 32-bit loads.  Correct for any alignment; not tuned.
+// thread with 32-bit loads, test-then-set.  Correct for any alignment; not tuned.
 template <int R>
 __global__ void __launch_bounds__(256)
 k_update_unaligned(const uint32_t *__restrict__ pairs, uint64_t n, uint32_t *__restrict__ grid,
@@ -187,7 +187,7 @@ k_update_unaligned(const uint32_t *__restrict__ pairs, uint64_t n, uint32_t *__r
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const Filter f{nullptr, 0};
     for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride)
-        apply_pair<R, 0>(grid, G, ld_stream_u32(pairs + 2 * t), ld_stream_u32(pairs + 2 * t + 1), true, f);
+        apply_pair<R, 1>(grid, G, ld_stream_u32(pairs + 2 * t), ld_stream_u32(pairs + 2 * t + 1), true, f);
 }
 
 template <int R, int MODE, int UNROLL>

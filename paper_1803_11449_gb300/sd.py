@@ -403,9 +403,9 @@ def sd_partition_pairs(h: Handle, direction: int, pairs, parts: int, out) -> np.
 
 
 def sd_update_noalloc(p: sd_params, grid, pairs, stream=None) -> int:
-    """Binned update into a caller-owned device DHLA `grid` (torch tensor of
+    """Update in place of a caller-owned device DHLA `grid` (torch tensor of
     dirs * sd_grid_words(p) 4-byte words) with no device allocation; returns
-    the C status code.  See include/sd.h for the scratch rules."""
+    the C status code.  See include/sd.h."""
     gptr, _, _g = _buffer(grid)
     ptr, n, _keep = _buffer(pairs)
     s = None if stream is None else (stream if isinstance(stream, int) else stream.cuda_stream)
