@@ -232,18 +232,21 @@ __device__ __forceinline__ void estimate_warp(const Geometry &G, const RestoreAr
 // A warp's buffered candidates to K, and their SZ and hits at once (the
 // estimators are hot, so in the DHLA; the loads hide behind other warps'
 // tests).  Hits of a direction whose K overflows are dropped by the host.
-__device__ __forceinline__ void flush_cands(const Geometry &G, const RestoreArgs &A, uint32_t dir, int szmax,
+// Returns whether K has passed its capacity (with every slot of K taken).
+__device__ __forceinline__ bool flush_cands(const Geometry &G, const RestoreArgs &A, uint32_t dir, int szmax,
                                             uint32_t *cbuf, unsigned long long *hbuf, uint32_t &ccount,
                                             uint32_t lane) {
-    if (ccount == 0) return;
+    if (ccount == 0) return false;
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(&A.stats->ncand[dir], (unsigned long long)ccount);
     base = __shfl_sync(0xFFFFFFFFu, base, 0);
     for (uint32_t q = lane; q < ccount; q += 32)
         if (base + q < A.cand_cap) A.cand[(uint64_t)dir * A.cand_cap + base + q] = cbuf[q];
-    if (base < A.cand_cap) estimate_warp(G, A, dir, szmax, cbuf, ccount, hbuf, lane);
+    const bool over = base + ccount > A.cand_cap;
+    if (!over) estimate_warp(G, A, dir, szmax, cbuf, ccount, hbuf, lane);
     ccount = 0;
     __syncwarp();
+    return over;
 }
 
 // 32-bit load from shared memory at byte address `addr`.
@@ -307,53 +310,52 @@ __device__ __forceinline__ bool restore_first(const RestoreConsts &C, uint32_t c
 }
 
 // Per-warp buffers of a block's restore.
+constexpr uint32_t kColumn = 16;  // survivors a lane may hold: two for each of kColumn / 2 c0 values
 struct WarpBufs {
-    uint2 *queue;              // [96] (a, c0) that passed the first stage
+    uint32_t *column;          // [kColumn][32] a lane's addresses that passed the first stage
     uint32_t *cand;            // [kWarpBuf] members of K
     unsigned long long *hits;  // [kWarpBuf]
-    uint32_t nqueue, ncand;    // (the same in every lane)
+    uint32_t ncand;            // (the same in every lane)
+    bool over;                 // K has passed its capacity: nothing more to find
 };
 
-// The second stage for the last n <= 32 queued addresses, one per lane.
-template <int R, int KM, int ALPHA, bool SMEM>
-__device__ __forceinline__ void restore_second(const Geometry &G, const RestoreArgs &A, const RestoreConsts &C,
-                                               uint32_t dir, int szmax, WarpBufs &W, uint32_t n, uint32_t lane) {
-    __syncwarp();
-    W.nqueue -= n;
-    const uint2 v = lane < n ? W.queue[W.nqueue + lane] : make_uint2(0u, 0u);
-    const bool in = lane < n && rows_hot<KM == kAbove16 ? 2 : 3, R, KM, ALPHA, SMEM>(C, v.x, v.y);
-    const unsigned b = __ballot_sync(0xFFFFFFFFu, in);
-    if (in) W.cand[W.ncand + __popc(b & ((1u << lane) - 1u))] = v.x;
-    W.ncand += __popc(b);
-    __syncwarp();
-    if (W.ncand >= 32) flush_cands(G, A, dir, szmax, W.cand, W.hits, W.ncand, lane);
-}
-
 // The tests of two (c1, t) items per thread against the tile's c0 values.
-// Few pass the first stage, so a lane's survivor waits in the warp's queue
-// and the other rows are looked up 32 survivors at a time.  Bound by
-// instruction issue (68%).  Measured with the estimates that follow in the
-// same launch, against all rows at once and a launch of its own for the
-// estimates: core sketch, 18 M tests, 77,000 candidates 51 us (56 and the
-// gap); k = 18, 168 M tests 357 us (598 + 15).
+// Few pass the first stage, so a lane puts its survivors in a column of its
+// own and the warp looks up the other rows for all columns after every eight
+// c0 values.  Bound by instruction issue (65%).  Measured with the estimates
+// that follow in the same launch, against all rows at once and a launch of
+// its own for the estimates: core sketch, 18 M tests, 77,000 candidates 48 us
+// (56 and the gap); k = 18, 168 M tests 307 us (598 + 15); 64 core sketches
+// 90 us (108 + 25); a window with every estimator hot, where each warp stops
+// as it sees K pass its capacity, close 1.1 ms less.
 template <int R, int KM, int ALPHA, bool SMEM>
 __device__ __forceinline__ void restore_x2(const Geometry &G, const RestoreArgs &A, const RestoreConsts &C,
                                            uint32_t dir, int szmax, const uint32_t *s_c0, uint32_t nc0, uint32_t c1a,
                                            uint32_t ta, bool va, uint32_t c1b, uint32_t tb, bool vb, WarpBufs &W,
                                            uint32_t lane) {
     const unsigned below = (1u << lane) - 1u;
-    for (uint32_t q = 0; q < nc0; q++) {
-        const uint32_t c0 = s_c0[q];  // same for the whole block
-        uint32_t aa, ab;
-        const bool fa = restore_first<R, KM, ALPHA, SMEM>(C, c0, c1a, ta, aa) && va;
-        const bool fb = restore_first<R, KM, ALPHA, SMEM>(C, c0, c1b, tb, ab) && vb;
-        const unsigned ba = __ballot_sync(0xFFFFFFFFu, fa), bb = __ballot_sync(0xFFFFFFFFu, fb);
-        if (!(ba | bb)) continue;
-        if (fa) W.queue[W.nqueue + __popc(ba & below)] = make_uint2(aa, c0);
-        W.nqueue += __popc(ba);
-        if (fb) W.queue[W.nqueue + __popc(bb & below)] = make_uint2(ab, c0);
-        W.nqueue += __popc(bb);
-        while (W.nqueue >= 32) restore_second<R, KM, ALPHA, SMEM>(G, A, C, dir, szmax, W, 32, lane);
+    uint32_t *const col = W.column + lane;
+    for (uint32_t q0 = 0; q0 < nc0 && !W.over; q0 += kColumn / 2) {
+        const uint32_t q1 = min(q0 + kColumn / 2, nc0);
+        uint32_t n = 0;
+#pragma unroll 4
+        for (uint32_t q = q0; q < q1; q++) {
+            const uint32_t c0 = s_c0[q];  // same for the whole block
+            uint32_t a;
+            if (restore_first<R, KM, ALPHA, SMEM>(C, c0, c1a, ta, a) && va) col[32u * n++] = a;
+            if (restore_first<R, KM, ALPHA, SMEM>(C, c0, c1b, tb, a) && vb) col[32u * n++] = a;
+        }
+        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n);
+        for (uint32_t j = 0; j < most; j++) {
+            const uint32_t a = j < n ? col[32u * j] : 0u;
+            const bool in = j < n && rows_hot<KM == kAbove16 ? 2 : 3, R, KM, ALPHA, SMEM>(C, a, dh0(C.A0, C.k, a));
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, in);
+            if (!b) continue;
+            if (in) W.cand[W.ncand + __popc(b & below)] = a;
+            W.ncand += __popc(b);
+            __syncwarp();
+            if (W.ncand >= 32 && flush_cands(G, A, dir, szmax, W.cand, W.hits, W.ncand, lane)) W.over = true;
+        }
     }
 }
 
@@ -376,55 +378,67 @@ __host__ __device__ __forceinline__ uint32_t restore_tile0(unsigned long long te
     const unsigned long long per = tests / ((unsigned long long)num_sms * 8u * kRestoreThreads * tiles_per_block) + 1;
     return (uint32_t)(per < kRestoreTileMax ? per : kRestoreTileMax);
 }
-__host__ __device__ __forceinline__ unsigned long long restore_tiles(const Geometry &G, uint32_t n0, uint32_t n1,
-                                                                     uint32_t tile0) {
+// (n1 <= 2^k items of 2^(32-2k) t: below 2^27; tiles: at most 2^31, as tile0
+// grows with the tests up to 256)
+__host__ __device__ __forceinline__ uint32_t restore_tiles(const Geometry &G, uint32_t n0, uint32_t n1,
+                                                           uint32_t tile0) {
     if (!n0 || !n1) return 0;
-    const unsigned long long items = (unsigned long long)n1 << restore_ulog(G);
-    return (unsigned long long)((n0 + tile0 - 1) / tile0) * ((items + kRestoreItems - 1) / kRestoreItems);
+    const uint32_t items = n1 << restore_ulog(G);
+    return ((n0 + tile0 - 1) / tile0) * ((items + kRestoreItems - 1) / kRestoreItems);
 }
 
 // The tiles first, first + step, ... below stop of one direction (see
-// restore_body), by one way of testing.
+// restore_body), by one way of testing.  A tile's lists are loaded while the
+// tile before it is tested.
 template <int R, int KM, int ALPHA, bool SMEM>
 __device__ __forceinline__ void restore_loop(const Geometry &G, const RestoreArgs &A, const RestoreConsts &C,
-                                             uint32_t dir, const RestoreDir &D, uint64_t first, uint64_t stop,
-                                             uint64_t step, WarpBufs &W, uint32_t *s_c0, bool *s_stop) {
+                                             uint32_t dir, const RestoreDir &D, uint32_t first, uint32_t stop,
+                                             uint32_t step, WarpBufs &W, uint32_t (*s_c0)[kRestoreTileMax],
+                                             bool *s_stop) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t *he0 = A.he + (uint64_t)dir * 2 * (1ull << G.k);
     const uint32_t *he1 = he0 + (1ull << G.k);
-    const uint64_t J = (uint64_t)D.n1 << C.ulog;
-    const uint64_t nchunk = (J + kRestoreItems - 1) / kRestoreItems;
-    // tile t covers c0 group t / nchunk and item chunk t % nchunk, stepped
-    // without dividing again
-    uint64_t t0 = first / nchunk, jc = first % nchunk;
-    const uint64_t t0_step = step / nchunk, jc_step = step % nchunk;
-    const uint32_t tm = (1u << C.ulog) - 1u;
-    for (uint64_t t = first; t < stop; t += step) {
-        const uint32_t c0_base = (uint32_t)t0 * D.tile0;
-        const uint32_t nc0 = min(D.tile0, D.n0 - c0_base);
-        // two (c1, t) items per thread
-        const uint64_t ja = jc * kRestoreItems + threadIdx.x, jb = ja + kRestoreThreads;
-        const bool va = ja < J, vb = jb < J;
-        const uint32_t c1a = va ? he1[ja >> C.ulog] : 0u, c1b = vb ? he1[jb >> C.ulog] : 0u;
+    const uint32_t J = D.n1 << C.ulog;
+    const uint32_t nchunk = (J + kRestoreItems - 1) / kRestoreItems;
+    // tile t covers c0 group t / nchunk and item chunk t % nchunk
+    uint32_t t0 = first / nchunk, jc = first % nchunk;
+    const uint32_t t0_step = step / nchunk, jc_step = step % nchunk, tm = (1u << C.ulog) - 1u;
+    // the next tile's c1 values (two (c1, t) items per thread), its c0 value
+    // of this thread, and whether K has passed its capacity: once it has, the
+    // direction reports nothing but the overload, and the rest of its
+    // enumeration is skipped (the same decision for the whole block; a warp
+    // that sees it earlier, as it adds to K, skips the rest of its tile)
+    uint32_t c1a = 0, c1b = 0, c0 = 0, ja = 0;
+    unsigned long long nk = 0;
+    auto load = [&]() {
+        ja = jc * kRestoreItems + threadIdx.x;
+        const uint32_t q = t0 * D.tile0 + threadIdx.x;
+        c1a = ja < J ? __ldcg(he1 + (ja >> C.ulog)) : 0u;
+        c1b = ja + kRestoreThreads < J ? __ldcg(he1 + ((ja + kRestoreThreads) >> C.ulog)) : 0u;
+        c0 = threadIdx.x < D.tile0 && q < D.n0 ? __ldcg(he0 + q) : 0u;
+        if (threadIdx.x == 0) nk = *reinterpret_cast<volatile unsigned long long *>(&A.stats->ncand[dir]);
+    };
+    load();
+    uint32_t cur = 0;
+    for (uint32_t t = first; t < stop;) {
+        s_c0[cur][threadIdx.x] = c0;
+        if (threadIdx.x == 0) s_stop[cur] = nk > A.cand_cap;
         __syncthreads();
-        // once K has passed its capacity the direction reports nothing but
-        // the overload, so the rest of its enumeration is skipped (one read
-        // of the shared counter per tile, the same decision for the block)
-        if (threadIdx.x == 0)
-            *s_stop = *reinterpret_cast<volatile unsigned long long *>(&A.stats->ncand[dir]) > A.cand_cap;
-        for (uint32_t q = threadIdx.x; q < nc0; q += kRestoreThreads) s_c0[q] = he0[c0_base + q];
-        __syncthreads();
-        if (*s_stop) break;
-        restore_x2<R, KM, ALPHA, SMEM>(G, A, C, dir, D.szmax, s_c0, nc0, c1a, (uint32_t)ja & tm, va, c1b,
-                                       (uint32_t)jb & tm, vb, W, lane);
+        if (s_stop[cur]) break;
+        const uint32_t nc0 = min(D.tile0, D.n0 - t0 * D.tile0);
+        const uint32_t xa = c1a, xb = c1b, xj = ja;
+        t += step < stop - t ? step : stop - t;  // (no wrap)
         t0 += t0_step;
         jc += jc_step;
         if (jc >= nchunk) {
             jc -= nchunk;
             t0++;
         }
+        if (t < stop) load();
+        restore_x2<R, KM, ALPHA, SMEM>(G, A, C, dir, D.szmax, s_c0[cur], nc0, xa, xj & tm, xj < J, xb,
+                                       (xj + kRestoreThreads) & tm, xj + kRestoreThreads < J, W, lane);
+        cur ^= 1u;
     }
-    if (W.nqueue) restore_second<R, KM, ALPHA, SMEM>(G, A, C, dir, D.szmax, W, W.nqueue, lane);
     __syncwarp();
     flush_cands(G, A, dir, D.szmax, W.cand, W.hits, W.ncand, lane);
 }
@@ -434,16 +448,16 @@ __device__ __forceinline__ void restore_loop(const Geometry &G, const RestoreArg
 // (worth it for more than a few tests per thread), where they fit.
 template <int R>
 __device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArgs &A, uint32_t dir, RestoreDir D,
-                                             bool stage, uint64_t t_begin, uint64_t t_end, uint64_t t_step) {
+                                             bool stage, uint32_t t_begin, uint32_t t_end, uint32_t t_step) {
     extern __shared__ uint32_t smem[];
     __shared__ unsigned long long s_hbuf[kRestoreThreads / 32][kWarpBuf];
     __shared__ uint32_t s_cbuf[kRestoreThreads / 32][kWarpBuf];
-    __shared__ uint2 s_queue[kRestoreThreads / 32][96];
-    __shared__ uint32_t s_c0[kRestoreTileMax];
-    __shared__ bool s_stop;
+    __shared__ uint32_t s_column[kRestoreThreads / 32][kColumn * 32];
+    __shared__ uint32_t s_c0[2][kRestoreTileMax];  // (kRestoreTileMax = kRestoreThreads)
+    __shared__ bool s_stop[2];
     __syncthreads();  // shared memory may still be in use by a previous call
-    const uint64_t ntiles = restore_tiles(G, D.n0, D.n1, D.tile0);
-    const uint64_t t_stop = t_end < ntiles ? t_end : ntiles;
+    const uint32_t ntiles = restore_tiles(G, D.n0, D.n1, D.tile0);
+    const uint32_t t_stop = t_end < ntiles ? t_end : ntiles;
     if (t_begin >= t_stop) return;  // no tile of this direction for the block
     RestoreConsts C;
     C.k = G.k;
@@ -457,6 +471,10 @@ __device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArg
     C.alpha = G.alpha;
     C.hot2 = A.hotmap + ((uint64_t)dir * G.r + 2u) * C.nw;
     C.hot2s = (uint32_t)__cvta_generic_to_shared(smem);
+    // kept in registers: the compiler would form them again from the kernel
+    // parameters in every test
+    asm volatile("" : "+r"(C.A0), "+r"(C.A0inv_k), "+r"(C.kmask), "+r"(C.lowbits), "+r"(C.lowmask), "+r"(C.k),
+                      "+r"(C.hot2s), "+r"(C.ulog));
     if (stage) {
         const uint32_t words = (G.r - 2) * C.nw;
         if ((C.nw & 3u) == 0) {  // (rows of whole 16-byte words: k >= 7)
@@ -469,9 +487,9 @@ __device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArg
         }
     }
     const uint32_t wid = threadIdx.x >> 5;
-    WarpBufs W{s_queue[wid], s_cbuf[wid], s_hbuf[wid], 0u, 0u};
+    WarpBufs W{s_column[wid], s_cbuf[wid], s_hbuf[wid], 0u, false};
 #define SD_RESTORE(KM, ALPHA, SMEM) \
-    restore_loop<R, KM, ALPHA, SMEM>(G, A, C, dir, D, t_begin, t_stop, t_step, W, s_c0, &s_stop)
+    restore_loop<R, KM, ALPHA, SMEM>(G, A, C, dir, D, t_begin, t_stop, t_step, W, s_c0, s_stop)
     if (stage) {
         if (R == 4 && G.k == 16u && G.alpha == 8u) SD_RESTORE(kIs16, 8, true);  // the core-link sketch
         else if (G.k == 16u) SD_RESTORE(kIs16, 0, true);
@@ -534,12 +552,12 @@ k_restore(const __grid_constant__ Geometry G, const __grid_constant__ RestoreArg
     // an L2 round trip per row: stage from two tests per thread on
     const bool stage = A.smem_hot && tests > (unsigned long long)gridDim.x * kRestoreThreads * 2u;
     const uint32_t tile0 = restore_tile0(tests, num_sms, 4);
-    uint64_t tiles0 = 0;
+    uint32_t skip = 0;  // blocks that direction 0's tiles end on
     for (uint32_t d = 0; d < G.dirs; d++) {
         const RestoreDir D{s_n[d][0], s_n[d][1], tile0, s_szmax[d]};
-        const uint64_t first = ((uint64_t)blockIdx.x + gridDim.x - tiles0 % gridDim.x) % gridDim.x;
-        restore_body<R>(G, A, d, D, stage, first, ~0ull, gridDim.x);
-        tiles0 += restore_tiles(G, D.n0, D.n1, D.tile0);
+        const uint32_t first = blockIdx.x >= skip ? blockIdx.x - skip : blockIdx.x + gridDim.x - skip;
+        restore_body<R>(G, A, d, D, stage, first, 0xFFFFFFFFu, gridDim.x);
+        skip = restore_tiles(G, D.n0, D.n1, D.tile0) % gridDim.x;
     }
 }
 
@@ -1079,8 +1097,8 @@ k_restore_many(const CloseJob *__restrict__ J, const unsigned long long *__restr
         const uint64_t end = tile_base[sg + 1] < b ? tile_base[sg + 1] : b;
         const CloseJob &j = J[sg >> 1];
         const RestoreDir D{j.A.n0[d], j.A.n1[d], j.A.tile0, j.A.szmax[d]};
-        restore_body<R>(j.G, j.A, d, D, j.A.smem_hot && (end - a) * D.tile0 > 2u, a - tile_base[sg],
-                        end - tile_base[sg], 1);
+        restore_body<R>(j.G, j.A, d, D, j.A.smem_hot && (end - a) * D.tile0 > 2u, (uint32_t)(a - tile_base[sg]),
+                        (uint32_t)(end - tile_base[sg]), 1u);
         a = end;
     }
 }

@@ -431,12 +431,9 @@ k_plane_scan(FoldJob one, const FoldJob *__restrict__ jobs, Geometry G, uint32_t
             z += __shfl_xor_sync(mask, z, o);
             nh += __shfl_xor_sync(mask, nh, o);
         }
-        __threadfence();  // every lane's bitmap word, before the row's count
-        __syncwarp(mask);
         if (w == 0) {
             atomicAdd(&job.st->zr[d][i], (unsigned long long)z);
             if (nh) atomicAdd(&job.st->nhot[d][i], nh);
-            s_list = i < 2 && atomicAdd(&job.st->rows_done[d][i], 1u) == wgroups - 1;
         }
     }
     __syncthreads();
@@ -458,6 +455,16 @@ k_plane_scan(FoldJob one, const FoldJob *__restrict__ jobs, Geometry G, uint32_t
         for (uint32_t j = 0; j < 32; j++, p += ps)
             if (any >> j & 1u) *p = 0u;
     }
+    if (i >= 2) return;
+    // rows 0 and 1: the block that counts the row's last estimators lists it
+    // (its bitmap words were written by the W threads above)
+    if (threadIdx.x < W) {
+        __threadfence();
+        constexpr uint32_t mask = W == 32 ? 0xFFFFFFFFu : (1u << W) - 1u;
+        __syncwarp(mask);
+        if (threadIdx.x == 0) s_list = atomicAdd(&job.st->rows_done[d][i], 1u) == wgroups - 1;
+    }
+    __syncthreads();
     if (s_list) {
         __threadfence();
         list_hot(job.hotmap + ((uint64_t)d * G.r + i) * rw, rw, job.he + ((uint64_t)d * 2 + i) * (1ull << G.k));
