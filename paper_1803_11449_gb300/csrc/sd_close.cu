@@ -526,6 +526,8 @@ k_restore(const __grid_constant__ Geometry G, const __grid_constant__ RestoreArg
           uint32_t num_sms) {
     __shared__ uint32_t s_n[2][2];
     __shared__ int s_szmax[2];
+    dependents_may_start();
+    wait_for_previous();
     if (threadIdx.x < 16) {  // eight lanes per direction, one row each
         const uint32_t d = threadIdx.x >> 3, i = threadIdx.x & 7u;
         const bool live = d < G.dirs && i < G.r;
@@ -668,6 +670,7 @@ k_close_finish(const unsigned long long *__restrict__ hits, uint64_t hits_cap, S
     __shared__ uint32_t s_cut[2], s_n, s_below;
     __shared__ bool s_last;
     const uint32_t dir = blockIdx.y;
+    wait_for_previous();
     const unsigned long long nh = st->nhits[dir];
     const bool fits = nh <= hits_cap && nh <= kFinishMax;
     const uint32_t n = fits ? (uint32_t)nh : 0u;
@@ -1194,15 +1197,15 @@ cudaError_t launch_restore(const Geometry &G, RestoreArgs A, uint64_t pair_cap, 
     if (e != cudaSuccess) return e;
     uint32_t sms = (uint32_t)num_sms;
     void *args[] = {const_cast<Geometry *>(&G), &A, &pair_cap, &xfac, &sms};
-    return cudaLaunchKernel(kern, dim3((unsigned)(num_sms * per_sm)), dim3(kRestoreThreads), args, smem, s);
+    return launch_dependent(kern, dim3((unsigned)(num_sms * per_sm)), dim3(kRestoreThreads), smem, s, args);
 }
 
 cudaError_t launch_close_finish(const unsigned long long *hits, uint64_t hits_cap, StatBlock *st,
                                 unsigned long long *out, uint64_t out_cap, unsigned long long *spare,
                                 StatBlock *st_out, uint32_t dirs, cudaStream_t s) {
-    k_close_finish<<<dim3(kFinishBlocks, dirs), kFinishThreads, 0, s>>>(hits, hits_cap, st, out, out_cap, spare,
-                                                                        st_out);
-    return cudaGetLastError();
+    void *args[] = {&hits, &hits_cap, &st, &out, &out_cap, &spare, &st_out};
+    return launch_dependent(reinterpret_cast<const void *>(k_close_finish), dim3(kFinishBlocks, dirs),
+                            dim3(kFinishThreads), 0, s, args);
 }
 
 cudaError_t launch_estimate(const Geometry &G, const RestoreArgs &A, int num_sms, cudaStream_t s) {

@@ -214,6 +214,27 @@ __device__ __forceinline__ uint32_t ld_weak(const uint32_t *p) {
     return v;
 }
 
+// Programmatic dependent launch: a kernel launched with launch_dependent is
+// set up while the kernel before it in the stream still runs, as soon as all
+// of that one's blocks have started (dependents_may_start) or ended.  It
+// touches nothing in memory before wait_for_previous, which returns once the
+// previous kernel is complete and its writes are visible.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+inline cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 // Launch set-up shared by every launcher: opts the kernel in to `smem` bytes
 // of dynamic shared memory when above 48 KiB and returns its resident blocks
 // per SM for (threads, smem).  Both are looked up once per (kernel, device,

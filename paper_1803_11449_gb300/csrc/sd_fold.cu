@@ -350,6 +350,7 @@ k_plane_scan(FoldJob one, const FoldJob *__restrict__ jobs, Geometry G, uint32_t
     __shared__ uint32_t s_part[7][S][W];
     __shared__ uint32_t s_hot[W];
     __shared__ bool s_list;
+    dependents_may_start();
     const uint32_t rw = (1u << G.k) >> 5;
     const uint32_t wgroups = (rw + W - 1) / W;
     uint32_t tile = blockIdx.x;

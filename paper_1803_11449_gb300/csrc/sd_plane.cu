@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArgs P, uint32_t head,
             uint32_t tile) {
     constexpr int E = PPT * DIRS;
+    dependents_may_start();
     extern __shared__ unsigned long long sm64[];
     __shared__ uint32_t s_warp[32];
     __shared__ bool s_last;
@@ -449,6 +450,7 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
     // unit (2^26 pairs of the core sketch: 270 us, 280 with searches and a
     // shared unit counter; 128 KiB planes, one block per SM: 345 and 362).
     const uint32_t x0 = blockIdx.x * per_block;
+    wait_for_previous();
     const uint32_t total = P.unit_start[NB];
     for (uint32_t b = threadIdx.x; b < NB; b += THREADS) {
         const uint32_t u0 = P.unit_start[b], u1 = P.unit_start[b + 1];
@@ -624,8 +626,10 @@ static cudaError_t launch_plane_apply(const Geometry &G, const PlaneArgs &P, uin
     const uint32_t nbuf = two && per_block > 1 ? 2u : 1u;
     const uint64_t blocks = (most + per_block - 1) / per_block;
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    kern<<<(unsigned)blocks, threads, plane * nbuf, s>>>(G, P, nbuf, (uint32_t)per_block);
-    return cudaGetLastError();
+    uint32_t nb = nbuf, pb = (uint32_t)per_block;
+    void *args[] = {const_cast<Geometry *>(&G), const_cast<PlaneArgs *>(&P), &nb, &pb};
+    return launch_dependent(reinterpret_cast<const void *>(kern), dim3((unsigned)blocks), dim3(threads), plane * nbuf, s,
+                            args);
 }
 
 cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
