@@ -720,10 +720,11 @@ static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
 // Algorithm 1 binned by plane over n device pairs of h, in rounds of at
 // most `round` pairs through `bins` (bin_words of them, at least the bins
 // of one round), on stream s; failures are reported on `rep`.  A round
-// reuses the layout the previous round of the same directions left when it
-// is no larger than that round and that layout fits the bins; a round of
-// another size is laid out from the previous counts scaled to its size when
-// that round had enough pairs; any other round is counted exactly.
+// reuses the layout the previous round of the same directions left, for a
+// longer round times a power of two (where that round had enough pairs to go
+// by), when that fits the bins; else it is laid out from the previous counts
+// scaled to its size (a launch of one block, 5 us, where bins are tight);
+// any other round is counted exactly.
 static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir, uint32_t *bins,
                         uint64_t bin_words, uint64_t round, cudaStream_t s, sd_handle *rep) {
     Geometry G = h->G;
@@ -749,8 +750,16 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
         }
         const uint64_t prev = h->plane_layout_view == dir ? h->plane_prev_pairs : 0;
         PlaneLayout L = kLayoutCount;
-        if (prev && m <= prev && plane_bin_words(G, prev) <= bin_words) L = kLayoutReuse;
-        else if (prev >= kPlaneScaleMinPerPlane * G.g) L = kLayoutScale;
+        P.shift = 0;
+        const bool usable = prev >= kPlaneScaleMinPerPlane * G.g;
+        if (prev && m > prev && usable)
+            while ((prev << P.shift) < m) P.shift++;
+        if (prev && (m <= prev || usable) && plane_bin_words(G, prev) << P.shift <= bin_words) {
+            L = kLayoutReuse;
+        } else {
+            P.shift = 0;
+            if (usable) L = kLayoutScale;
+        }
         SD_CK(rep, launch_plane_round(pairs + 2 * off, m, G, P, h->num_sms, s, L, prev));
         launched(L == kLayoutReuse ? 2 : 3);
         h->plane_prev_pairs = m;

@@ -66,6 +66,7 @@ struct PlaneArgs {
     uint32_t ps;           // words per plane: r 2^k / 32 rounded up to 4
     uint32_t unit;         // entries per apply unit (a multiple of 4)
     uint32_t tile_pairs;   // pairs per binning tile
+    uint32_t shift;        // the round's bins: binoff and cap times 2^shift
 };
 
 // One link of a batched binned update (device memory table).
@@ -298,6 +299,9 @@ size_t plane_bin_smem_bytes(uint32_t tile_pairs, uint32_t dirs, uint32_t nbins);
 // How a plane round gets its bin layout: the one the previous round left
 // (its counts plus slack), that round's counts scaled by n / prev_pairs
 // (plus slack), or an exact count of this round's keys.
+// kLayoutReuse with P.shift > 0 takes the previous round's bins times a
+// power of two: a longer round needs no launch for its layout where the bins
+// have that room.
 enum PlaneLayout { kLayoutReuse = 0, kLayoutScale = 1, kLayoutCount = 2 };
 cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
                                cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs);

@@ -127,6 +127,10 @@ __device__ __forceinline__ void write_layout(const PlaneArgs &P, bool slack, uin
     }
 }
 
+// First slot and slots of plane b's bin in this round.
+__device__ __forceinline__ uint32_t bin_off(const PlaneArgs &P, uint32_t b) { return P.binoff[b] << P.shift; }
+__device__ __forceinline__ uint32_t bin_room(const PlaneArgs &P, uint32_t b) { return P.cap[b] << P.shift; }
+
 // The last block to call this (one call per block, counter at *done) gets
 // true, after a fence that makes every earlier block's writes visible.
 __device__ __forceinline__ bool last_block(uint32_t *done, bool *s_last) {
@@ -357,8 +361,8 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
                 offs[b] = run;
                 if (h) {
                     res[q] = atomicAdd(&P.cnt[b], h);
-                    rcap[q] = P.cap[b];
-                    roff[q] = P.binoff[b];
+                    rcap[q] = bin_room(P, b);
+                    roff[q] = bin_off(P, b);
                 }
                 hist[b] = 0;
                 run += h;
@@ -368,8 +372,8 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
             const uint32_t h = hist[b];
             offs[b] = run;
             if (h) {
-                const uint32_t pos = atomicAdd(&P.cnt[b], h), c = P.cap[b];
-                dst[b] = make_uint2(P.binoff[b] + pos - run, run + (c > pos ? c - pos : 0u));
+                const uint32_t pos = atomicAdd(&P.cnt[b], h), c = bin_room(P, b);
+                dst[b] = make_uint2(bin_off(P, b) + pos - run, run + (c > pos ? c - pos : 0u));
             }
             hist[b] = 0;
             run += h;
@@ -407,7 +411,7 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
     // the last block: apply units of the bins' actual contents
     if (!last_block(&P.ctl[0], &s_last)) return;
     const uint32_t U = P.unit;
-    block_scan(NB, [&](uint32_t i) { return (min(__ldcg(&P.cnt[i]), P.cap[i]) + U - 1u) / U; },
+    block_scan(NB, [&](uint32_t i) { return (min(__ldcg(&P.cnt[i]), bin_room(P, i)) + U - 1u) / U; },
                [&](uint32_t i, uint32_t v) { P.unit_start[i] = v; }, s_warp);
     if (threadIdx.x == 0) {
         P.ctl[0] = 0;
@@ -455,7 +459,7 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
     for (uint32_t b = threadIdx.x; b < NB; b += THREADS) {
         const uint32_t u0 = P.unit_start[b], u1 = P.unit_start[b + 1];
         if (u1 <= x0 || u0 >= x0 + per_block) continue;
-        const uint32_t off = P.binoff[b], n = min(P.cnt[b], P.cap[b]);
+        const uint32_t off = bin_off(P, b), n = min(P.cnt[b], bin_room(P, b));
 #pragma unroll
         for (uint32_t j = 0; j < kApplyUnitsPerBlock; j++) {
             const uint32_t x = x0 + j;

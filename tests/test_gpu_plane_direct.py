@@ -63,3 +63,14 @@ def test_both_sides_of_the_line_in_one_window(mods, sketch, offset):
     win = T.make_window(w, 4, n=1_700_003).pairs
     # the line lies between 0.47 M (paper) and 0.9 M (tiny) pairs
     _check(mods, w, [win, win[:333], win[5:1_500_002], win[7:1_000_008], win[9:200_010]], offset)
+
+
+def test_growing_rounds_and_shifted_traffic(mods):
+    """Rounds of 0.8 M, 1.7 M, 3.3 M and 1.6 M pairs: bins of the round before
+    times 1, 2 and 4, and traffic whose planes they do not fit."""
+    w = T.WORKLOADS["core"].with_(src_pool=1 << 16, dst_pool=1 << 18, planted=0)
+    win = T.make_window(w, 6, n=3_300_001).pairs
+    other = win.copy()
+    other[::2] = other[0]  # half of the pairs in one plane of either direction
+    _check(mods, w, [win[:800_001], win[5:1_700_000], other, win[: 1_600_000]], 0)
+    _check(mods, w, [win[:800_001], other, win], 2)
