@@ -1,8 +1,9 @@
 // sd_fold.cu -- the fold of the plane-binned update's plane-major DHLA copy
 // into the estimator-major DHLA (grid |= planes^T, then planes = 0), run
-// before anything reads the DHLA: the window close (one launch for every
-// handle of a batched close), sd_get_grid, sd_set_grid, sd_merge,
-// sd_export_grid and sd_or_grid.
+// before anything reads the DHLA: sd_get_grid, sd_set_grid, sd_merge,
+// sd_export_grid, sd_or_grid and the window close (one launch for every
+// handle of a batched close) -- except a close whose DHLA is the plane copy
+// alone, which counts the copy as it is (k_plane_scan below).
 //
 // Plane (d, b) holds bit b of every estimator of direction d: its row i
 // starts at word i * 2^k/32 and holds estimator c's bit at word c >> 5, bit

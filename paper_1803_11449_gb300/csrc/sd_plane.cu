@@ -18,12 +18,16 @@
 //                  slack; keys beyond a bin's capacity (traffic that shifted
 //                  between rounds) set their bits directly with atomic ORs.
 //                  The last block cuts each plane's bin into apply units.
-//   k_plane_layout for a round of another size than the previous one (of
-//                  enough pairs to go by): that round's per-plane counts
-//                  scaled to this round's size, plus slack.
+//                  A longer round than the one before (of enough pairs to
+//                  go by) takes those bins times a power of two.
+//   k_plane_layout for a longer round where the bins have not that room:
+//                  the previous per-plane counts scaled to this round's
+//                  size, plus slack.
 //   k_plane_count  for a round with no usable history (the first one, one
 //                  over other directions, or one after a small round): the
 //                  exact keys of every plane, and a layout without slack.
+//   k_plane_direct for a round of few pairs, instead of all the others: every
+//                  bit ORed into the plane copy where it lies.
 //   k_plane_apply  one unit (a plane and a range of its bin) per block step:
 //                  the plane in shared memory, DH_0 and Eq. 2 of every key,
 //                  r shared-memory ORs, then one bulk OR of the plane into
@@ -31,9 +35,11 @@
 //                  (cp.reduce.async.bulk ... .or.b32, so units of one plane
 //                  may run on several SMs).  The last block lays out the
 //                  next round's bins from this round's counts.
-//   k_plane_fold   (sd_fold.cu; window close, sd_get_grid, sd_merge) folds
-//                  the plane-major copy into the estimator-major DHLA
-//                  (grid |= planes^T) and clears it.
+//   k_plane_scan   (sd_fold.cu; window close) counts the plane-major copy as
+//                  it is and clears it.
+//   k_plane_fold   (sd_fold.cu; sd_get_grid, sd_merge, and a close where the
+//                  DHLA holds bits of its own) folds the copy into the
+//                  estimator-major DHLA (grid |= planes^T) and clears it.
 //
 // Per pair this moves dirs keys (4 bytes each) through the bins instead of
 // r * dirs bit positions, and the plane copy is swept once per round by
