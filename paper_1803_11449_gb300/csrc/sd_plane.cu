@@ -261,7 +261,9 @@ __device__ __forceinline__ void bin_hash(uint32_t cnt, const uint32_t (&ps)[PPT]
     }
 }
 
-template <int DIRS, int PPT, int THREADS>
+// SHIFTED: the round's bins are the layout times 2^P.shift (a kernel of its
+// own: the shifts cost the others 3% through the register allocation).
+template <int DIRS, int PPT, int THREADS, bool SHIFTED>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArgs P, uint32_t head,
             uint32_t tile) {
@@ -367,8 +369,8 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
                 offs[b] = run;
                 if (h) {
                     res[q] = atomicAdd(&P.cnt[b], h);
-                    rcap[q] = bin_room(P, b);
-                    roff[q] = bin_off(P, b);
+                    rcap[q] = SHIFTED ? bin_room(P, b) : P.cap[b];
+                    roff[q] = SHIFTED ? bin_off(P, b) : P.binoff[b];
                 }
                 hist[b] = 0;
                 run += h;
@@ -378,8 +380,8 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
             const uint32_t h = hist[b];
             offs[b] = run;
             if (h) {
-                const uint32_t pos = atomicAdd(&P.cnt[b], h), c = bin_room(P, b);
-                dst[b] = make_uint2(bin_off(P, b) + pos - run, run + (c > pos ? c - pos : 0u));
+                const uint32_t pos = atomicAdd(&P.cnt[b], h), c = SHIFTED ? bin_room(P, b) : P.cap[b];
+                dst[b] = make_uint2((SHIFTED ? bin_off(P, b) : P.binoff[b]) + pos - run, run + (c > pos ? c - pos : 0u));
             }
             hist[b] = 0;
             run += h;
@@ -417,7 +419,7 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
     // the last block: apply units of the bins' actual contents
     if (!last_block(&P.ctl[0], &s_last)) return;
     const uint32_t U = P.unit;
-    block_scan(NB, [&](uint32_t i) { return (min(__ldcg(&P.cnt[i]), bin_room(P, i)) + U - 1u) / U; },
+    block_scan(NB, [&](uint32_t i) { return (min(__ldcg(&P.cnt[i]), SHIFTED ? bin_room(P, i) : P.cap[i]) + U - 1u) / U; },
                [&](uint32_t i, uint32_t v) { P.unit_start[i] = v; }, s_warp);
     if (threadIdx.x == 0) {
         P.ctl[0] = 0;
@@ -574,7 +576,7 @@ size_t plane_bin_smem_bytes(uint32_t tile_pairs, uint32_t dirs, uint32_t nbins) 
 template <int DIRS, int PPT, int THREADS>
 static cudaError_t launch_plane_bin(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P,
                                     uint32_t head, int num_sms, cudaStream_t s) {
-    auto kern = k_plane_bin<DIRS, PPT, THREADS>;
+    auto kern = P.shift ? k_plane_bin<DIRS, PPT, THREADS, true> : k_plane_bin<DIRS, PPT, THREADS, false>;
     const size_t smem = plane_bin_smem_bytes(P.tile_pairs, DIRS, P.nbins);
     int per_sm = 0;
     cudaError_t e = prepare_launch(reinterpret_cast<const void *>(kern), THREADS, smem, &per_sm);
