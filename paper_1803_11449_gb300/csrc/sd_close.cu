@@ -1300,7 +1300,8 @@ cudaError_t launch_restore_many(const CloseJob *J, const CloseJob *Jh, uint32_t 
                                 unsigned long long *tile_base_h, int num_sms, cudaStream_t s, int *launches) {
     *launches = 0;
     const Geometry &G = Jh[0].G;
-    const size_t smem = Jh[0].A.smem_hot ? restore_hot_bytes(G) : 16;
+    // (of the shape: a job that does not run has no smem_hot of its own)
+    const size_t smem = restore_hot_bytes(G) <= kRestoreHotMax ? restore_hot_bytes(G) : 16;
     unsigned long long acc = 0;
     bool any = false;
     for (uint32_t i = 0; i < count; i++) {
