@@ -105,6 +105,9 @@ k_plane_fold(FoldJob one, const FoldJob *__restrict__ jobs, uint32_t njobs, Geom
     const uint64_t per_job = (uint64_t)G.dirs * G.r * wgroups * tgroups;
     const uint64_t tiles = per_job * njobs;
     const uint32_t W4 = W / 4, rows = 32u * TC;
+    // rows of one or two words (k < 7) have no 16-byte words: copied and
+    // cleared word by word
+    const uint32_t words = W4 ? 0u : rows * W;
     const uint32_t tt = threadIdx.x / W, w = threadIdx.x % W;
     const uint32_t lane = threadIdx.x & 31u;
     // a tile's first plane word
@@ -117,6 +120,12 @@ k_plane_fold(FoldJob one, const FoldJob *__restrict__ jobs, uint32_t njobs, Geom
             const FoldTile f = fold_tile(tile, per_job, tgroups, wgroups, TC, W, G, one, jobs);
             const uint32_t *pb = plane_base(f);
             const uint32_t sa = (uint32_t)__cvta_generic_to_shared(stage0 + s * kFoldTile);
+            for (uint32_t q = threadIdx.x; q < words; q += blockDim.x) {
+                const uint32_t row = q / W, c = q - row * W;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                             ::"r"(sa + 4u * q), "l"(pb + (uint64_t)row * ps + c)
+                             : "memory");
+            }
             for (uint32_t q = threadIdx.x; q < rows * W4; q += blockDim.x) {
                 const uint32_t row = q / W4, c = q - row * W4;
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
@@ -141,6 +150,10 @@ k_plane_fold(FoldJob one, const FoldJob *__restrict__ jobs, uint32_t njobs, Geom
         uint32_t *in = stage0 + cur * kFoldTile;
         // clear the tile's plane words that hold bits
         uint32_t *pb = plane_base(f);
+        for (uint32_t q = threadIdx.x; q < words; q += blockDim.x) {
+            const uint32_t row = q / W, c = q - row * W;
+            if (in[q]) pb[(uint64_t)row * ps + c] = 0u;
+        }
         for (uint32_t q = threadIdx.x; q < rows * W4; q += blockDim.x) {
             const uint4 v = reinterpret_cast<const uint4 *>(in)[q];
             if (v.x | v.y | v.z | v.w) {
