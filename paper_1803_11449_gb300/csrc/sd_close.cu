@@ -210,10 +210,10 @@ __device__ __forceinline__ void estimate_warp(const Geometry &G, const RestoreAr
                     const uint32_t ci = i == 0 ? c0 : ((shr_clamp(x, (i - 1u) * G.alpha) & kmask) ^ c0);
                     const uint32_t *cell = gdir + (uint64_t)i * G.row_words + (uint64_t)ci * G.wpc;
                     if (wide) {
-                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(cell) + c);
+                        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(cell) + c);
                         ule.x &= v.x; ule.y &= v.y; ule.z &= v.z; ule.w &= v.w;
                     } else {
-                        ule.x &= __ldg(cell + c);
+                        ule.x &= __ldcg(cell + c);
                     }
                 }
                 ones += __popc(ule.x) + __popc(ule.y) + __popc(ule.z) + __popc(ule.w);
@@ -662,9 +662,8 @@ __device__ __forceinline__ uint32_t count_below(const uint32_t *v, uint32_t n, u
 }
 
 __global__ void __launch_bounds__(kFinishThreads)
-k_close_finish(const unsigned long long *__restrict__ hits, uint64_t hits_cap, StatBlock *st,
-               unsigned long long *__restrict__ out, uint64_t out_cap, unsigned long long *__restrict__ spare,
-               StatBlock *st_out) {
+k_close_finish(const unsigned long long *hits, uint64_t hits_cap, StatBlock *st, unsigned long long *out,
+               uint64_t out_cap, unsigned long long *spare, StatBlock *st_out) {
     __shared__ unsigned long long s_key[kRangeKeys];
     __shared__ __align__(16) uint32_t s_ip[kRangeKeys + 4];
     __shared__ uint32_t s_cut[2], s_n, s_below;
@@ -693,7 +692,7 @@ k_close_finish(const unsigned long long *__restrict__ hits, uint64_t hits_cap, S
             // come out eight times as long, one of 512 four times)
             const uint32_t per = n <= 32768u ? 2u : 4u, m = per * nb;
             for (uint32_t i = threadIdx.x; i < ((m + 3u) & ~3u); i += kFinishThreads)
-                s_ip[i] = i < m ? (uint32_t)(h[(uint64_t)i * n / m] >> 32) : ~0u;
+                s_ip[i] = i < m ? (uint32_t)(__ldcg(h + (uint64_t)i * n / m) >> 32) : ~0u;
             __syncthreads();
             for (uint32_t i = threadIdx.x; i < m; i += kFinishThreads) {
                 const uint32_t x = s_ip[i], rank = count_below(s_ip, m, x);

@@ -219,9 +219,19 @@ __device__ __forceinline__ uint32_t ld_weak(const uint32_t *p) {
 // set up while the kernel before it in the stream still runs, as soon as all
 // of that one's blocks have started (dependents_may_start) or ended.  It
 // touches nothing in memory before wait_for_previous, which returns once the
-// previous kernel is complete and its writes are visible.
+// previous kernel is complete and its writes are visible.  What the previous
+// kernel wrote is read with coherent loads (plain, __ldcg or ld_previous_v4):
+// .nc loads, __ldg and const __restrict__ need data that stays the same from
+// the start of the reading kernel.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ uint4 ld_previous_v4(const uint4 *p) {
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
 inline cudaError_t launch_dependent(const void *kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args) {
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

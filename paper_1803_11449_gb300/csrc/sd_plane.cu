@@ -495,7 +495,7 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
         for (; q + 3 * blockDim.x < n4; q += 4 * blockDim.x) {
             uint4 v[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) v[j] = ld_stream_v4(e4 + q + j * blockDim.x);
+            for (int j = 0; j < 4; j++) v[j] = ld_previous_v4(e4 + q + j * blockDim.x);
 #pragma unroll
             for (int j = 0; j < 4; j++) {
                 apply_key<R>(pl, G, A0, rw, v[j].x); apply_key<R>(pl, G, A0, rw, v[j].y);
@@ -503,12 +503,12 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
             }
         }
         for (; q < n4; q += blockDim.x) {
-            const uint4 a = ld_stream_v4(e4 + q);
+            const uint4 a = ld_previous_v4(e4 + q);
             apply_key<R>(pl, G, A0, rw, a.x); apply_key<R>(pl, G, A0, rw, a.y);
             apply_key<R>(pl, G, A0, rw, a.z); apply_key<R>(pl, G, A0, rw, a.w);
         }
         for (uint32_t r = beg + 4 * n4 + threadIdx.x; r < end; r += blockDim.x)
-            apply_key<R>(pl, G, A0, rw, ld_stream_u32(P.bins + r));
+            apply_key<R>(pl, G, A0, rw, __ldcg(P.bins + r));
         __syncthreads();
         if (threadIdx.x == 0) {
             // the plane's bits into the plane-major DHLA copy, ORed in L2
