@@ -310,7 +310,7 @@ k_bin(const uint32_t *__restrict__ pairs, uint64_t n, uint32_t *__restrict__ gri
 
 __global__ void __launch_bounds__(1024)
 k_apply(uint32_t *__restrict__ grid, BinArgs B, const LinkDesc *__restrict__ links, uint32_t slices_per_link) {
-    extern __shared__ uint32_t slice[];
+    extern __shared__ __align__(16) uint32_t slice[];
     __shared__ uint32_t s_cur;
     const uint32_t SW = 1u << B.slice_log2;
     for (;;) {

@@ -449,7 +449,8 @@ __device__ __forceinline__ void restore_loop(const Geometry &G, const RestoreArg
 template <int R>
 __device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArgs &A, uint32_t dir, RestoreDir D,
                                              bool stage, uint32_t t_begin, uint32_t t_end, uint32_t t_step) {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ uint4 smem4[];  // (filled in 16-byte words)
+    uint32_t *const smem = reinterpret_cast<uint32_t *>(smem4);
     __shared__ unsigned long long s_hbuf[kRestoreThreads / 32][kWarpBuf];
     __shared__ uint32_t s_cbuf[kRestoreThreads / 32][kWarpBuf];
     __shared__ uint32_t s_column[kRestoreThreads / 32][kColumn * 32];
@@ -478,7 +479,7 @@ __device__ __forceinline__ void restore_body(const Geometry &G, const RestoreArg
     if (stage) {
         const uint32_t words = (G.r - 2) * C.nw;
         if ((C.nw & 3u) == 0) {  // (rows of whole 16-byte words: k >= 7)
-            uint4 *to = reinterpret_cast<uint4 *>(smem);
+            uint4 *to = smem4;
             const uint4 *from = reinterpret_cast<const uint4 *>(C.hot2);
 #pragma unroll 4
             for (uint32_t w = threadIdx.x; w < words / 4; w += kRestoreThreads) to[w] = __ldcg(from + w);
