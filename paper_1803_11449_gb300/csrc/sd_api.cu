@@ -288,12 +288,16 @@ struct sd_handle {
     }
 };
 
+// A failed call's error is taken out of the runtime's per-thread state, where
+// the next launch would find it and report it as its own.
 #define SD_CK(h, call)                                                                         \
     do {                                                                                       \
         cudaError_t e_ = (call);                                                               \
-        if (e_ != cudaSuccess)                                                                 \
+        if (e_ != cudaSuccess) {                                                               \
+            cudaGetLastError();                                                                \
             return (h)->fail(e_ == cudaErrorMemoryAllocation ? SD_ERR_NOMEM : SD_ERR_CUDA,     \
                              "%s: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__, __LINE__); \
+        }                                                                                      \
     } while (0)
 
 namespace sd {
