@@ -1296,11 +1296,25 @@ static int queue_restore(sd_handle *h, float xfac) {
     return SD_OK;
 }
 
+// The staged join's buffers, before a close touches the window: one that
+// cannot have them returns with the window as it was.
+static int ensure_join(sd_handle *h) {
+    const Geometry &G = h->G;
+    h->join_cap = 4 * h->cand_cap;
+    if (!h->he_all) SD_CK(h, cudaMalloc(&h->he_all, ((uint64_t)G.dirs * G.r << G.k) * 4));
+    if (!h->jsub) SD_CK(h, cudaMalloc(&h->jsub, 2 * G.dirs * h->join_cap * 8));
+    return SD_OK;
+}
+
 static int close_phase_a(sd_handle *h, sd_report *out) {
     std::memset(out, 0, sizeof *out);
     std::memset(&h->cs, 0, sizeof h->cs);
     h->report.clear();
     h->last_ncand[0] = h->last_ncand[1] = 0;
+    if (h->T.restore == 1) {
+        const int jrc = ensure_join(h);
+        if (jrc != SD_OK) return jrc;
+    }
     if (h->planes_dirty && fold_stats_fit(h->G) && (h->grid_clean || h->grid_stale)) {
         // the whole DHLA is the plane copy: counted as it is
         const FoldJob job{h->grid, h->planes, 1u, h->zhot, h->st_d, h->hotmap, h->he};
@@ -1378,11 +1392,6 @@ static int close_phase_b(sd_handle *h, sd_report *out) {
     RestoreArgs &A = h->cs.A;
     h->cs.queued_b = h->T.restore == 1;
     if (h->T.restore == 1) {
-        if (!h->jsub) {
-            h->join_cap = 4 * h->cand_cap;
-            SD_CK(h, cudaMalloc(&h->he_all, ((uint64_t)G.dirs * G.r << G.k) * 4));
-            SD_CK(h, cudaMalloc(&h->jsub, 2 * G.dirs * h->join_cap * 8));
-        }
         JoinArgs J;
         std::memset(&J, 0, sizeof J);
         J.he = h->he_all;

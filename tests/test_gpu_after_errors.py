@@ -56,3 +56,36 @@ def test_out_of_memory_is_reported_once(mods, mode):
         _same(O, op, og, sd.sd_close_window(h))
     finally:
         sd.sd_destroy(h)
+
+
+def test_a_close_without_memory_for_the_join_keeps_the_window(mods):
+    """2^31 candidates: the handle's lists take 86 GB, the staged join's 275 GB.
+    The close that cannot have them leaves the window as it was, alone and
+    among others."""
+    torch, sd, O = mods
+    torch.cuda.empty_cache()
+    w = T.WORKLOADS["core"].with_(n=1 << 17, src_pool=1 << 14, dst_pool=1 << 14, planted=4,
+                                  planted_c=("uniform", 1500, 4000))
+    wins = [T.make_window(w, s).pairs for s in (1, 2)]
+    op = O.params_from(w.sketch(), seed=SEED)
+    grids = [O.new_grid(op) for _ in wins]
+    for og, pairs in zip(grids, wins):
+        O.update(op, og, pairs)
+    h, h2 = sd.sd_create(sd.params_for(w, SEED, cand_cap=1 << 31)), sd.sd_create(sd.params_for(w, SEED))
+    try:
+        for window in range(2):
+            sd.sd_set_tuning(h, mode=6, restore=1)
+            sd.sd_update(h, _dev(torch, wins[0]))
+            with pytest.raises(sd.SdError) as e:
+                sd.sd_close_window(h)
+            assert e.value.code == -2  # SD_ERR_NOMEM
+            sd.sd_update(h2, _dev(torch, wins[1]))
+            with pytest.raises(sd.SdError):
+                sd.sd_close_many([h, h2])
+            sd.sd_set_tuning(h, mode=6, restore=0)
+            _same(O, op, grids[0], sd.sd_close_window(h))
+            rep = sd.sd_close_window(h2)  # closed above, beside the one that failed
+            assert rep.n_hits_total == 0 and rep.psi == [0.0, 0.0]
+    finally:
+        sd.sd_destroy(h)
+        sd.sd_destroy(h2)
