@@ -44,15 +44,16 @@ def test_out_of_memory_is_reported_once(mods, mode):
     op = O.params_from(w.sketch(), seed=SEED)
     og = O.new_grid(op)
     O.update(op, og, pairs)
+    dev = _dev(torch, pairs)
     h = sd.sd_create(sd.params_for(w, SEED))
     try:
         with pytest.raises(sd.SdError):  # 2^40 candidates: 4 TiB
             sd.sd_create(sd.params_for(w, SEED, cand_cap=1 << 40))
         sd.sd_set_tuning(h, mode=5, bin_chunk_log2=28, bin_slack_pct=40000)  # bins of terabytes
         with pytest.raises(sd.SdError):
-            sd.sd_update(h, _dev(torch, pairs))
+            sd.sd_update(h, dev)
         sd.sd_set_tuning(h, mode=mode, bin_chunk_log2=20, bin_slack_pct=100)
-        sd.sd_update(h, _dev(torch, pairs))
+        sd.sd_update(h, dev)
         _same(O, op, og, sd.sd_close_window(h))
     finally:
         sd.sd_destroy(h)
@@ -71,15 +72,16 @@ def test_a_close_without_memory_for_the_join_keeps_the_window(mods):
     grids = [O.new_grid(op) for _ in wins]
     for og, pairs in zip(grids, wins):
         O.update(op, og, pairs)
+    dev = [_dev(torch, pairs) for pairs in wins]  # (kept until their updates are done)
     h, h2 = sd.sd_create(sd.params_for(w, SEED, cand_cap=1 << 31)), sd.sd_create(sd.params_for(w, SEED))
     try:
         for window in range(2):
             sd.sd_set_tuning(h, mode=6, restore=1)
-            sd.sd_update(h, _dev(torch, wins[0]))
+            sd.sd_update(h, dev[0])
             with pytest.raises(sd.SdError) as e:
                 sd.sd_close_window(h)
             assert e.value.code == -2  # SD_ERR_NOMEM
-            sd.sd_update(h2, _dev(torch, wins[1]))
+            sd.sd_update(h2, dev[1])
             with pytest.raises(sd.SdError):
                 sd.sd_close_many([h, h2])
             sd.sd_set_tuning(h, mode=6, restore=0)

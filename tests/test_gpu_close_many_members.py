@@ -21,15 +21,16 @@ def test_members_behind_one_that_does_not_restore(first, O):
     wins = [T.make_window(w, s).pairs for s in (21, 22, 23)]
     seeds = [210, 220, 230]
     caps = [dict(pair_cap=1) if first == "overloaded" else {}, {}, {}]
+    dev = [torch.from_numpy(p.reshape(-1).view(np.int32)).cuda() for p in wins]  # (kept until the closes)
     hs = [sd.sd_create(sd.params_for(w, s, **c)) for s, c in zip(seeds, caps)]
     ops = [O.params_from(w.sketch(), seed=s, **c) for s, c in zip(seeds, caps)]
     try:
         for window in range(2):
             grids = []
-            for i, (h, op, pairs) in enumerate(zip(hs, ops, wins)):
+            for i, (h, op, pairs, on) in enumerate(zip(hs, ops, wins, dev)):
                 og = O.new_grid(op)
                 if i or first != "empty":
-                    sd.sd_update(h, torch.from_numpy(pairs.reshape(-1).view(np.int32)).cuda())
+                    sd.sd_update(h, on)
                     O.update(op, og, pairs)
                 if i == 0 and first == "saturated":
                     full = np.full(og.size // 2, 0xFFFFFFFF, np.uint32)
