@@ -201,8 +201,8 @@ struct sd_handle {
     unsigned long long *hits_tmp = nullptr;  // [dirs][hits_cap]: scratch of the large-list sort
     unsigned long long *hits_h = nullptr; // pinned [2][finish_cap]: ordered hits
     uint64_t finish_cap = 0;
+    std::unique_ptr<unsigned long long[]> hits_spill[2];  // a list that no pinned memory could be had for
     uint64_t cand_cap = 0, hits_cap = 0, report_cap = 0, pair_cap = 0;
-    unsigned long long *big_h = nullptr;  // pinned [2][hits_cap]: large sorted hit lists
     void *ss_d = nullptr;                 // [2] sample-sort scratch (kSampleScratchBytes each)
     uint32_t *ss_flag_h = nullptr;        // pinned [2]: a sample sort fell short
     bool ss_check[2] = {false, false};    // ss_flag_h[d] is to be checked after the close's last sync
@@ -492,7 +492,6 @@ static void release(sd_handle *h) {
     cudaFreeHost(h->fj_h);
     cudaFreeHost(h->st_h);
     cudaFreeHost(h->hits_h);
-    cudaFreeHost(h->big_h);
     cudaFree(h->ss_d);
     cudaFreeHost(h->ss_flag_h);
     for (int b = 0; b < 2; b++) {
@@ -1438,22 +1437,28 @@ static int close_phase_c(sd_handle *h, sd_report *out, bool *need_sync) {
     CloseState &c = h->cs;
     *need_sync = false;
     h->ss_check[0] = h->ss_check[1] = false;
-    // lists that were ordered but did not fit hits_h: a larger one, for this
-    // close and the next ones (any list already in the old one moves along)
+    // lists that do not fit hits_h: a larger one, for this close and the next
+    // ones (any list already in the old one moves along).  By now the window
+    // is out of the DHLA, so memory that cannot be had must not lose it: such
+    // a list goes to pageable memory.
     uint64_t want = 0;
     for (uint32_t d = 0; d < h->G.dirs; d++)
-        if (c.A.run[d] && h->st_h->big_sort[d] == 2) want = std::max<uint64_t>(want, h->st_h->nhits[d]);
+        if (c.A.run[d] && h->st_h->big_sort[d] && h->st_h->ncand[d] <= h->cand_cap)
+            want = std::max<uint64_t>(want, h->st_h->nhits[d]);
     if (want > h->finish_cap) {
         const uint64_t cap = next_pow2(want);
         unsigned long long *grown = nullptr;
-        SD_CK(h, cudaMallocHost(&grown, (uint64_t)2 * cap * 8));
-        for (uint32_t d = 0; d < h->G.dirs; d++)
-            if (c.A.run[d] && h->st_h->big_sort[d] == 0)
-                std::memcpy(grown + d * cap, h->hits_h + d * h->finish_cap,
-                            std::min<uint64_t>(h->st_h->nhits[d], h->finish_cap) * 8);
-        cudaFreeHost(h->hits_h);
-        h->hits_h = grown;
-        h->finish_cap = cap;
+        if (cudaMallocHost(&grown, (uint64_t)2 * cap * 8) == cudaSuccess) {
+            for (uint32_t d = 0; d < h->G.dirs; d++)
+                if (c.A.run[d] && h->st_h->big_sort[d] == 0)
+                    std::memcpy(grown + d * cap, h->hits_h + d * h->finish_cap,
+                                std::min<uint64_t>(h->st_h->nhits[d], h->finish_cap) * 8);
+            cudaFreeHost(h->hits_h);
+            h->hits_h = grown;
+            h->finish_cap = cap;
+        } else {
+            cudaGetLastError();
+        }
     }
     for (uint32_t d = 0; d < h->G.dirs; d++) {
         if (!c.A.run[d]) continue;
@@ -1474,30 +1479,33 @@ static int close_phase_c(sd_handle *h, sd_report *out, bool *need_sync) {
         c.nh[d] = h->st_h->nhits[d];
         c.keys[d] = h->hits_h + (uint64_t)d * h->finish_cap;
         if (!h->st_h->big_sort[d]) continue;
-        if (h->st_h->big_sort[d] == 2) {
-            SD_CK(h, cudaMemcpyAsync(h->hits_h + (uint64_t)d * h->finish_cap, h->hits_tmp + (uint64_t)d * h->hits_cap,
-                                     c.nh[d] * 8, cudaMemcpyDeviceToHost, h->stream));
-            *need_sync = true;
-            continue;
+        unsigned long long *dst = h->hits_h + (uint64_t)d * h->finish_cap;
+        if (c.nh[d] > h->finish_cap) {
+            h->hits_spill[d].reset(new (std::nothrow) unsigned long long[c.nh[d]]);
+            if (!h->hits_spill[d]) return h->fail(SD_ERR_NOMEM, "sd_close_window: no memory for %llu hits",
+                                                  (unsigned long long)c.nh[d]);
+            dst = h->hits_spill[d].get();
         }
-        unsigned long long *sorted = nullptr;
-        uint32_t *overflow = nullptr;
-        int nl = 0;
-        if (!h->ss_d) {
-            SD_CK(h, cudaMalloc(&h->ss_d, 2 * kSampleScratchBytes));
-            SD_CK(h, cudaMallocHost(&h->ss_flag_h, 2 * sizeof(uint32_t)));
-        }
-        SD_CK(h, launch_sort_big(h->hits + (uint64_t)d * h->hits_cap, h->hits_tmp + (uint64_t)d * h->hits_cap,
-                                 c.nh[d], static_cast<char *>(h->ss_d) + d * kSampleScratchBytes, h->num_sms,
-                                 h->stream, &sorted, &nl, &overflow));
-        launched(nl);
-        if (!h->big_h) SD_CK(h, cudaMallocHost(&h->big_h, (uint64_t)2 * h->hits_cap * 8));
-        unsigned long long *dst = h->big_h + (uint64_t)d * h->hits_cap;
-        SD_CK(h, cudaMemcpyAsync(dst, sorted, c.nh[d] * 8, cudaMemcpyDeviceToHost, h->stream));
-        h->ss_check[d] = overflow != nullptr;
-        if (overflow)
-            SD_CK(h, cudaMemcpyAsync(h->ss_flag_h + d, overflow, 4, cudaMemcpyDeviceToHost, h->stream));
         c.keys[d] = dst;
+        const unsigned long long *sorted = h->hits_tmp + (uint64_t)d * h->hits_cap;
+        if (h->st_h->big_sort[d] != 2) {
+            unsigned long long *out_d = nullptr;
+            uint32_t *overflow = nullptr;
+            int nl = 0;
+            // (without scratch of its own: by sorted segments and merges)
+            if (!h->ss_flag_h && cudaMallocHost(&h->ss_flag_h, 2 * sizeof(uint32_t)) != cudaSuccess) cudaGetLastError();
+            if (h->ss_flag_h && !h->ss_d && cudaMalloc(&h->ss_d, 2 * kSampleScratchBytes) != cudaSuccess)
+                cudaGetLastError();
+            void *scratch = h->ss_d ? static_cast<char *>(h->ss_d) + d * kSampleScratchBytes : nullptr;
+            SD_CK(h, launch_sort_big(h->hits + (uint64_t)d * h->hits_cap, h->hits_tmp + (uint64_t)d * h->hits_cap,
+                                     c.nh[d], scratch, h->num_sms, h->stream, &out_d, &nl, &overflow));
+            launched(nl);
+            sorted = out_d;
+            h->ss_check[d] = overflow != nullptr;
+            if (overflow)
+                SD_CK(h, cudaMemcpyAsync(h->ss_flag_h + d, overflow, 4, cudaMemcpyDeviceToHost, h->stream));
+        }
+        SD_CK(h, cudaMemcpyAsync(dst, sorted, c.nh[d] * 8, cudaMemcpyDeviceToHost, h->stream));
         *need_sync = true;
     }
     return SD_OK;
@@ -1518,8 +1526,8 @@ static int redo_short_sorts(sd_handle *h) {
         SD_CK(h, launch_sort_big(h->hits + (uint64_t)d * h->hits_cap, h->hits_tmp + (uint64_t)d * h->hits_cap,
                                  c.nh[d], nullptr, h->num_sms, h->stream, &sorted, &nl, &overflow));
         launched(nl);
-        SD_CK(h, cudaMemcpyAsync(h->big_h + (uint64_t)d * h->hits_cap, sorted, c.nh[d] * 8, cudaMemcpyDeviceToHost,
-                                 h->stream));
+        SD_CK(h, cudaMemcpyAsync(const_cast<unsigned long long *>(c.keys[d]), sorted, c.nh[d] * 8,
+                                 cudaMemcpyDeviceToHost, h->stream));
         SD_CK(h, cudaStreamSynchronize(h->stream));
     }
     return SD_OK;
@@ -1802,7 +1810,7 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         bool b = false;
         rcs[i] = close_phase_c(h, &outs[i], &b);
         for (uint32_t dd = 0; dd < G.dirs; dd++)
-            if (h->cs.keys[dd] == h->hits_h + (uint64_t)dd * h->finish_cap)
+            if (h->cs.keys[dd] && !h->st_h->big_sort[dd])
                 h->cs.keys[dd] = d->cb_hits_h + ((uint64_t)i * 2 + dd) * kSortSmall;
         big[i] = b;
         any_big = any_big || b;
