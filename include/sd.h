@@ -224,7 +224,10 @@ int sd_update(sd_handle *h, const uint32_t *pairs, uint64_t n);
  * Blocks until the report is ready, then clears the DHLA (asynchronously, in
  * stream order).  Returns SD_OK, or SD_ERR_SATURATED / SD_ERR_OVERLOAD /
  * SD_ERR_REPORT_OVERFLOW with *out still filled (flags say which direction);
- * the window is closed in every one of these cases. */
+ * the window is closed in every one of these cases.  A close with the staged
+ * join (restore = 1) whose lists do not fit the device returns SD_ERR_NOMEM
+ * with the window as it was.  After any other hard error what the window held
+ * may be lost; the next window starts with clean counters. */
 int sd_close_window(sd_handle *h, sd_report *out);
 
 /* Close the windows of `count` handles at once: the same work and results

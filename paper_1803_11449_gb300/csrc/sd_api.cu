@@ -251,6 +251,7 @@ struct sd_handle {
     bool planes_dirty = false;
     bool grid_clean = false;           // the DHLA is all zero (reset, then plane updates only)
     bool grid_stale = false;           // the DHLA is empty but its words hold an earlier close's bits
+    bool stats_used = false;           // st_d may hold the counters of a close that did not end
     uint64_t plane_prev_pairs = 0;     // pairs of the round whose counts are in prev (0: none)
     int plane_layout_view = -2;        // its directions (-1 both, else one)
 
@@ -1295,6 +1296,15 @@ static int queue_restore(sd_handle *h, float xfac) {
     return SD_OK;
 }
 
+// The counters in st_d for a close on stream s.  Every close that ends leaves
+// them zero; one that returned early may have left its own, on which the next
+// one's would be added up (and HE(0) and HE(1) not be listed again).
+static int claim_stats(sd_handle *h, cudaStream_t s) {
+    if (h->stats_used) SD_CK(h, cudaMemsetAsync(h->st_d, 0, sizeof(StatBlock), s));
+    h->stats_used = true;
+    return SD_OK;
+}
+
 // The staged join's buffers, before a close touches the window: one that
 // cannot have them returns with the window as it was.
 static int ensure_join(sd_handle *h) {
@@ -1314,6 +1324,8 @@ static int close_phase_a(sd_handle *h, sd_report *out) {
         const int jrc = ensure_join(h);
         if (jrc != SD_OK) return jrc;
     }
+    const int crc = claim_stats(h, h->stream);
+    if (crc != SD_OK) return crc;
     if (h->planes_dirty && fold_stats_fit(h->G) && (h->grid_clean || h->grid_stale)) {
         // the whole DHLA is the plane copy: counted as it is
         const FoldJob job{h->grid, h->planes, 1u, h->zhot, h->st_d, h->hotmap, h->he};
@@ -1578,6 +1590,7 @@ static int close_phase_d(sd_handle *h, sd_report *out, bool reset = true) {
         launched(1);
         h->grid_clean = !h->planes_dirty;
     }
+    if (reset) h->stats_used = false;
 
     uint32_t flags = c.flags;
     out->n_hits_total = h->report.size();
@@ -1714,6 +1727,8 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
     bool any_fresh = false;
     for (uint32_t i = 0; i < count; i++) {
         sd_handle *h = hs[i];
+        const int crc = claim_stats(h, s);
+        if (crc != SD_OK) return crc;
         if (h->planes_dirty && fold_stats && (h->grid_clean || h->grid_stale)) folded[i] = 2, nscan++;
         else any_fresh = true;
     }
@@ -1824,7 +1839,10 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         if (rcs[i] == SD_OK) rcs[i] = close_phase_d(hs[i], &outs[i], false);
     SD_CK(d, launch_reset_many(d->cj_d, count, G, d->num_sms, s));
     launched(1);
-    for (uint32_t i = 0; i < count; i++) hs[i]->grid_clean = !hs[i]->grid_stale && !hs[i]->planes_dirty;
+    for (uint32_t i = 0; i < count; i++) {
+        hs[i]->grid_clean = !hs[i]->grid_stale && !hs[i]->planes_dirty;
+        hs[i]->stats_used = false;
+    }
     tr.mark(3);
     // each member's later work waits for the batch
     SD_CK(d, cudaEventRecord(d->ev_batch, s));
