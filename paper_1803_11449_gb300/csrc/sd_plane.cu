@@ -60,6 +60,8 @@ constexpr uint32_t kPlaneThreads = 512;   // k_plane_bin / k_plane_count block
 constexpr uint32_t kApplyThreads = 512;   // k_plane_apply block (1024 where one plane fills the block's shared memory)
 constexpr uint32_t kHeldReservations = 2;  // reservation results a thread holds across the scatter
 constexpr uint32_t kBinTilesPerBlock = 8;   // k_plane_bin tiles per block (blocks retire as a round runs)
+constexpr uint32_t kDirectThreads = 256;    // k_plane_direct block: a tile of pairs (numbered in 8 bits)
+constexpr uint32_t kDirectSlots = 2048;     // hash slots for finding a tile's equal pairs
 constexpr uint32_t kApplyUnitsPerBlock = 4; // k_plane_apply units per block, at most
 
 __device__ __forceinline__ uint32_t h1v(uint64_t A1, uint64_t B1, uint32_t lg, uint32_t y) {
@@ -532,29 +534,44 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
 // A short round: every key's bits ORed into the plane copy where they lie,
 // one pair per thread, with no bins and no planes in shared memory.  Bound
 // by the L2's random reductions; the binned round's floor is the sweep of
-// the whole plane copy through shared memory, whatever the pairs.  A pair
-// equal to its predecessor (a flow's packets in a burst) is skipped.
+// the whole plane copy through shared memory, whatever the pairs.
+//
+// Reductions of one word are taken one after another, so the packets of one
+// flow must not each bring theirs: of the equal pairs of a block's tile one is
+// set.  Each thread writes its number to the slot of its pair's hash, and
+// skips the pair when the slot then names another thread with an equal one
+// (a slot taken by a different pair lets all of the others through: with
+// 2048 slots, one block in twenty).  2^19 pairs, none, a fifth and half of
+// them one interleaved flow: tiny sketch 24, 22 and 19 us (every pair set but
+// a repeat of the one before it: 24, 121 and 179), core sketch 33, 29 and 24
+// (35, 93 and 129), 256 MiB copy 36, 35 and 31 (37, 210 and 294).
 template <int DIRS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kDirectThreads)
 k_plane_direct(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArgs P) {
+    __shared__ uint2 s_pair[kDirectThreads];
+    __shared__ uint8_t s_slot[kDirectSlots];
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const bool pair8 = ((uintptr_t)pairs & 7u) == 0;
     for (uint64_t p0 = (uint64_t)blockIdx.x * blockDim.x; p0 < n; p0 += stride) {
         const uint64_t p = p0 + threadIdx.x;
         const bool ok = p < n;
-        uint32_t s = 0, t = 0;
+        uint2 v = make_uint2(0u, 0u);
         if (ok && pair8) {
-            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(pairs) + p);
-            s = v.x;
-            t = v.y;
+            v = __ldg(reinterpret_cast<const uint2 *>(pairs) + p);
         } else if (ok) {
-            s = ld_stream_u32(pairs + 2 * p);
-            t = ld_stream_u32(pairs + 2 * p + 1);
+            v.x = ld_stream_u32(pairs + 2 * p);
+            v.y = ld_stream_u32(pairs + 2 * p + 1);
         }
-        const uint32_t us = __shfl_up_sync(0xFFFFFFFFu, s, 1), ut = __shfl_up_sync(0xFFFFFFFFu, t, 1);
-        if (!ok || ((threadIdx.x & 31u) && us == s && ut == t)) continue;
-        set_key_bits<DIRS>(G, P, h1v(G.h[0].A1, G.h[0].B1, G.lg, t), s);
-        if (DIRS == 2) set_key_bits<DIRS>(G, P, G.g + h1v(G.h[1].A1, G.h[1].B1, G.lg, s), t);
+        const uint32_t slot = (v.x * 0x9E3779B1u + v.y * 0x85EBCA6Bu) / (uint32_t)((1ull << 32) / kDirectSlots);
+        __syncthreads();  // the previous tile's look-ups are done
+        s_pair[threadIdx.x] = v;
+        if (ok) s_slot[slot] = (uint8_t)threadIdx.x;
+        __syncthreads();
+        const uint32_t first = s_slot[slot];
+        const uint2 f = s_pair[first];
+        if (!ok || (first != threadIdx.x && f.x == v.x && f.y == v.y)) continue;
+        set_key_bits<DIRS>(G, P, h1v(G.h[0].A1, G.h[0].B1, G.lg, v.y), v.x);
+        if (DIRS == 2) set_key_bits<DIRS>(G, P, G.g + h1v(G.h[1].A1, G.h[1].B1, G.lg, v.x), v.y);
     }
 }
 
@@ -562,9 +579,9 @@ cudaError_t launch_plane_direct(const uint32_t *pairs, uint64_t n, const Geometr
                                 cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     auto kern = G.dirs == 2 ? k_plane_direct<2> : k_plane_direct<1>;
-    uint64_t blocks = (n + 255) / 256;
+    uint64_t blocks = (n + kDirectThreads - 1) / kDirectThreads;
     if (blocks > (uint64_t)num_sms * 32) blocks = (uint64_t)num_sms * 32;
-    kern<<<(unsigned)blocks, 256, 0, s>>>(pairs, n, G, P);
+    kern<<<(unsigned)blocks, kDirectThreads, 0, s>>>(pairs, n, G, P);
     return cudaGetLastError();
 }
 
