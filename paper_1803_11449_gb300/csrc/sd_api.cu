@@ -248,12 +248,13 @@ struct sd_handle {
     uint64_t lane_bins_words[kBatchLanes - 1] = {};
     cudaEvent_t lane_ev[kBatchLanes] = {};
     PlaneArgs pa{};                    // counters and plane copy (bins, tile, unit set per round)
-    bool planes_dirty = false;
+    bool planes_dirty = false;         // the plane copy may hold bits
     bool grid_clean = false;           // the DHLA is all zero (reset, then plane updates only)
     bool grid_stale = false;           // the DHLA is empty but its words hold an earlier close's bits
     bool stats_used = false;           // st_d may hold the counters of a close that did not end
     uint64_t plane_prev_pairs = 0;     // pairs of the round whose counts are in prev (0: none)
     int plane_layout_view = -2;        // its directions (-1 both, else one)
+    bool plane_replays = false;        // rounds were captured into a graph: replays are not seen here
 
     // key partition (sd_partition_pairs): per-part counts and cursors
     unsigned long long *part_d = nullptr;  // [2][1024]
@@ -728,7 +729,8 @@ static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
 // longer round times a power of two (where that round had enough pairs to go
 // by), when that fits the bins; else it is laid out from the previous counts
 // scaled to its size (a launch of one block, 5 us, where bins are tight);
-// any other round is counted exactly.
+// any other round is counted exactly, as is every one of a handle whose rounds
+// are in a graph.
 static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir, uint32_t *bins,
                         uint64_t bin_words, uint64_t round, cudaStream_t s, sd_handle *rep) {
     Geometry G = h->G;
@@ -745,6 +747,14 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
     if (!plane_direct(G, n, round) && plane_bin_words(G, std::min(round, n)) > bin_words)
         return rep->fail(SD_ERR_ARG, "plane update: %llu bin words for rounds of %llu pairs",
                          (unsigned long long)bin_words, (unsigned long long)round);
+    // Which layout the device holds is known from the rounds queued here.  A
+    // graph with such rounds in it runs them again unseen, on whatever layout
+    // (of other directions, of a longer round) lies there by then: from the
+    // first captured round on, every round of the handle is counted and its
+    // plane copy is always taken to hold bits.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    SD_CK(rep, cudaStreamIsCapturing(s, &capture));
+    if (capture != cudaStreamCaptureStatusNone) h->plane_replays = true;
     for (uint64_t off = 0; off < n; off += round) {
         const uint64_t m = std::min(round, n - off);
         if (plane_direct(G, m, round)) {
@@ -752,7 +762,7 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
             launched(1);
             continue;
         }
-        const uint64_t prev = h->plane_layout_view == dir ? h->plane_prev_pairs : 0;
+        const uint64_t prev = h->plane_layout_view == dir && !h->plane_replays ? h->plane_prev_pairs : 0;
         PlaneLayout L = kLayoutCount;
         P.shift = 0;
         const bool usable = prev >= kPlaneScaleMinPerPlane * G.g;
@@ -791,7 +801,7 @@ static int fold_planes(sd_handle *h) {
     const FoldJob job{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot, nullptr, nullptr, nullptr};
     SD_CK(h, launch_plane_fold(job, nullptr, 1, h->G, h->pa.ps, h->num_sms, h->stream));
     launched(1);
-    h->planes_dirty = false;
+    h->planes_dirty = h->plane_replays;
     h->grid_clean = false;
     return SD_OK;
 }
@@ -1331,7 +1341,7 @@ static int close_phase_a(sd_handle *h, sd_report *out) {
         const FoldJob job{h->grid, h->planes, 1u, h->zhot, h->st_d, h->hotmap, h->he};
         SD_CK(h, launch_plane_scan(job, nullptr, 1, h->G, h->pa.ps, h->stream));
         launched(1);
-        h->planes_dirty = false;
+        h->planes_dirty = h->plane_replays;
         h->grid_clean = false;
         h->grid_stale = true;
     } else {
@@ -1340,7 +1350,7 @@ static int close_phase_a(sd_handle *h, sd_report *out) {
             const FoldJob job{h->grid, h->planes, h->grid_clean ? 1u : 0u, h->zhot, h->st_d, h->hotmap, nullptr};
             SD_CK(h, launch_plane_fold(job, nullptr, 1, h->G, h->pa.ps, h->num_sms, h->stream));
             launched(1);
-            h->planes_dirty = false;
+            h->planes_dirty = h->plane_replays;
             h->grid_clean = false;
         } else {
             const int frc = fold_planes(h);
@@ -1736,7 +1746,7 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
         sd_handle *h = hs[i];
         if (folded[i] == 2) {
             d->fj_h[at++] = FoldJob{h->grid, h->planes, 1u, h->zhot, h->st_d, h->hotmap, h->he};
-            h->planes_dirty = false;
+            h->planes_dirty = h->plane_replays;
             h->grid_clean = false;
             h->grid_stale = true;
         } else {
@@ -1749,7 +1759,7 @@ static int close_many_batched(sd_handle *const *hs, uint32_t count, sd_report *o
                                                fold_stats ? h->st_d : nullptr, fold_stats ? h->hotmap : nullptr,
                                                nullptr};
             folded[i] = fold_stats;
-            h->planes_dirty = false;
+            h->planes_dirty = h->plane_replays;
             h->grid_clean = false;
         }
     }
