@@ -157,10 +157,6 @@ k_compact(const uint32_t *__restrict__ hotmap, Geometry G, uint32_t *__restrict_
 }
 
 // ---------------------------------------------------------------- restore
-__device__ __forceinline__ bool hot_at(const uint32_t *bm_row, uint32_t c) {
-    return (bm_row[c >> 5] >> (c & 31u)) & 1u;
-}
-
 constexpr uint32_t kRestoreTileMax = 256;  // c0 values per k_restore tile
 
 // Per-warp output buffers of the restore: candidates and hits are reserved

@@ -60,7 +60,7 @@ struct PlaneArgs {
     uint32_t *binoff;      // [nbins + 1] first slot of each plane's bin
     uint32_t *cap;         // [nbins] slots of each plane's bin; keys beyond them are set directly
     uint32_t *unit_start;  // [nbins + 1] first apply unit of each plane
-    uint32_t *ctl;         // [0] blocks done (count or bin), [2] apply blocks done
+    uint32_t *ctl;         // [0] blocks done (count or bin), [1] apply blocks done
     uint32_t *planes;      // [nbins][ps] plane-major DHLA copy
     uint32_t nbins;        // dirs * g
     uint32_t ps;           // words per plane: r 2^k / 32 rounded up to 4

@@ -425,7 +425,7 @@ k_plane_bin(const uint32_t *__restrict__ pairs, uint64_t n, Geometry G, PlaneArg
                [&](uint32_t i, uint32_t v) { P.unit_start[i] = v; }, s_warp);
     if (threadIdx.x == 0) {
         P.ctl[0] = 0;
-        P.ctl[2] = 0;
+        P.ctl[1] = 0;
     }
 }
 
@@ -523,10 +523,11 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
         }
     }
     // (shared memory must outlive the reductions' reads; the reductions
-    // themselves are complete when the kernel is)
+    // themselves are complete when the kernel is: what reads the plane copy
+    // next is a plain launch, and must stay one)
     if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     // the last block: the next round's bins from this round's counts
-    if (!last_block(&P.ctl[2], &s_last)) return;
+    if (!last_block(&P.ctl[1], &s_last)) return;
     write_layout(P, true, s_warp);
 }
 
