@@ -138,7 +138,8 @@ typedef struct {
                                   Algorithm 1 sets in all r estimators of the key -- then
                                   each bit plane's estimators DH_i(key) set in shared
                                   memory and ORed into a plane-major copy of the DHLA,
-                                  folded into the DHLA before it is read */
+                                  folded into the DHLA before it is read
+                                  (a close may count the copy as it is) */
     uint32_t block_threads; /* threads per block: 64..1024, multiple of 32 */
     uint32_t blocks_per_sm; /* resident blocks per SM the grid is sized for (0: as
                                many as fit) */

@@ -636,12 +636,15 @@ k_sort_small(unsigned long long *hits, uint64_t hits_cap, StatBlock *st, uint2 r
 // same sample of 2 or 4 hits per range, and reads the whole list: it keeps the
 // hits of its range in shared memory and counts those below, which is where
 // its part of the order begins.  So no block waits for another and one
-// launch does it: 29,000 hits in 21 us and 2,400 in 12 us with cold caches,
+// launch does it: 29,000 hits in 24 us and 2,400 in 12 us with cold caches,
 // where the one-block sort and the sample sort's four launches took 42 and
 // 23 us and a host round trip.  Within a block a hit's place is the number
 // of smaller addresses (addresses are distinct).  A range with more than
 // kRangeKeys hits, or a list of more than kFinishMax, sets big_sort: the
-// host sorts it by the longer way.
+// host sorts it by the longer way.  A range of 2 or 4 sample gaps of 128 hits
+// on average is that long in one list of 4,000 at 32,768 hits (reckoned) and
+// one of 100 at 65,536 (16 of 1600 counted).  Twice the samples there take 62
+// us instead of 39 for every such launch, more than the rare longer way.
 constexpr uint32_t kFinishThreads = 1024;
 constexpr uint32_t kFinishLoads = 4;       // 16-byte loads in flight per thread
 constexpr uint32_t kFinishBlocks = 128;    // ranges at most

@@ -286,9 +286,9 @@ cudaError_t launch_plane_fold(const FoldJob &one, const FoldJob *jobs, uint32_t 
 // the hot test z_0 <= zhot, i.e. count >= g - zhot, is a bit-sliced
 // comparison.  No transpose, except of the 32 x 32 blocks whose word has a
 // hot estimator.  Bound by the plane copy's read and clear: the core
-// sketch's 32 MiB take 16 us with few hot estimators and 22 us with 4,200 a
+// sketch's 32 MiB take 14 us with few hot estimators and 22 us with 4,200 a
 // row (the fold with statistics, the lists and the DHLA's clear took 28 to
-// 33, 4 and 6.5 us); 64 of them 0.96 ms (1.4 and 0.3 ms), 4.5 TB/s.
+// 33, 4 and 6.5 us); 64 of them 0.94 ms (1.4 and 0.3 ms), 4.6 TB/s.
 constexpr uint32_t kScanThreads = 256;
 constexpr uint32_t kCountBits = 12;  // counts up to 1024
 
