@@ -717,9 +717,21 @@ static int ensure_plane_bins(sd_handle *owner, uint64_t words) {
 // 3 M bit-sets (2^20 pairs of a 0.5 MiB copy: 27 and 26 us) to 6 M (2^19.5
 // pairs of a 32 MiB copy: 33 and 37 us), and for a copy beyond L2 at 8 M to
 // 16 M (2^20 pairs of 256 MiB: 78 and 155 us; 2^21: 258 and 164 us).
+//
+// Planes of few words: a busy host's pairs all set bits of the one plane of
+// its H1 (two directions) or of its own few words (one), reductions of a word
+// are serialised, and a direct round takes 20 to 40 us per million bit-sets
+// instead of 5, while a binned one stays under 40 us.  They meet, for sources
+// drawn from 2^8 to 2^18 hosts by Zipf's law, two directions: 64-word planes
+// at 0.3 to 0.6 M bit-sets, 192 words 0.5 M, 512 words 0.8 to 1.2 M, 2048
+// words 2.2 M, 2560 words in a 20 MiB copy 3.6 M; one direction: 64 and 192
+// words 1 M, 512 words 3.3 M.  (64-word planes, 2^17 pairs, two directions:
+// 101 to 139 us direct and 46 binned.)
 static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
-    const uint64_t copy_words = (uint64_t)G.dirs * G.g * plane_words(G);
-    return m < round && m * G.dirs * G.r <= std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3);
+    const uint64_t ps = plane_words(G), copy_words = (uint64_t)G.dirs * G.g * ps;
+    const uint64_t narrow = G.dirs == 2 ? (5ull << 16) + 1024 * ps + copy_words / 8 : (5ull << 17) + 4096 * ps;
+    const uint64_t most = std::min(std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3), narrow);
+    return m < round && m * G.dirs * G.r <= most;
 }
 
 // Algorithm 1 binned by plane over n device pairs of h, in rounds of at
