@@ -60,6 +60,7 @@ constexpr uint32_t kPlaneThreads = 512;   // k_plane_bin / k_plane_count block
 constexpr uint32_t kApplyThreads = 512;   // k_plane_apply block (1024 where one plane fills the block's shared memory)
 constexpr uint32_t kHeldReservations = 2;  // reservation results a thread holds across the scatter
 constexpr uint32_t kBinTilesPerBlock = 8;   // k_plane_bin tiles per block (blocks retire as a round runs)
+constexpr uint32_t kDependentPlaneWords = 512;  // narrower planes: k_plane_apply in a plain launch
 constexpr uint32_t kDirectThreads = 256;    // k_plane_direct block: a tile of pairs (numbered in 8 bits)
 constexpr uint32_t kDirectSlots = 2048;     // hash slots for finding a tile's equal pairs
 constexpr uint32_t kApplyUnitsPerBlock = 4; // k_plane_apply units per block, at most
@@ -658,6 +659,14 @@ static cudaError_t launch_plane_apply(const Geometry &G, const PlaneArgs &P, uin
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     uint32_t nb = nbuf, pb = (uint32_t)per_block;
     void *args[] = {const_cast<Geometry *>(&G), const_cast<PlaneArgs *>(&P), &nb, &pb};
+    // Narrow planes: a unit's atomics meet on few words, and its block wants an
+    // SM of its own.  Set up beside k_plane_bin's blocks, several land on one
+    // (700,001 pairs in two directions, update alone: 64-word planes 96 us as
+    // dependents and 46 plain, 192 words 45 and 35; 512 words 34 and 36, 8192
+    // words 42 and 42, 2^21 pairs 54 and 56).
+    if (P.ps < kDependentPlaneWords)
+        return cudaLaunchKernel(reinterpret_cast<const void *>(kern), dim3((unsigned)blocks), dim3(threads), args,
+                                plane * nbuf, s);
     return launch_dependent(reinterpret_cast<const void *>(kern), dim3((unsigned)blocks), dim3(threads), plane * nbuf, s,
                             args);
 }
