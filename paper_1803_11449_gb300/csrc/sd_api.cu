@@ -720,16 +720,19 @@ static int ensure_plane_bins(sd_handle *owner, uint64_t words) {
 //
 // Planes of few words: a busy host's pairs all set bits of the one plane of
 // its H1 (two directions) or of its own few words (one), reductions of a word
-// are serialised, and a direct round takes 20 to 40 us per million bit-sets
-// instead of 5, while a binned one stays under 40 us.  They meet, for sources
-// drawn from 2^8 to 2^18 hosts by Zipf's law, two directions: 64-word planes
-// at 0.3 to 0.6 M bit-sets, 192 words 0.5 M, 512 words 0.8 to 1.2 M, 2048
-// words 2.2 M, 2560 words in a 20 MiB copy 3.6 M; one direction: 64 and 192
-// words 1 M, 512 words 3.3 M.  (64-word planes, 2^17 pairs, two directions:
-// 101 to 139 us direct and 46 binned.)
+// are serialised, and a direct round takes 10 to 40 us per million bit-sets
+// instead of 5.  Where they meet, in millions, measured for sources drawn from
+// 2^8, 2^12 and 2^18 hosts by Zipf's law (g, r, k): two directions 0.3 (32, 8,
+// 8), 0.65 (256, 8, 8), 1.3 (1024, 8, 8), 0.6 (64, 6, 10), 1.0 (512, 5, 11),
+// 1.0 (64, 4, 12), 0.85 to 1.1 (256, 4, 12), 1.3 to 1.9 (1024, 4, 12), 2.2
+// (512, 4, 14), 2.2 to 2.7 (256, 5, 14), 3.6 (1024, 5, 14); one direction 0.46
+// (32, 8, 8), 1.1 (256, 8, 8), 1.0 (64, 6, 10), 2.9 (256, 5, 11), 3.2 (256, 4,
+// 12).  `narrow` is a line near or below these.  (32, 8, 8 with 2^17 pairs and two
+// directions: 102 to 139 us direct and 40 binned.)
 static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
-    const uint64_t ps = plane_words(G), copy_words = (uint64_t)G.dirs * G.g * ps;
-    const uint64_t narrow = G.dirs == 2 ? (5ull << 16) + 1024 * ps + copy_words / 8 : (5ull << 17) + 4096 * ps;
+    const uint64_t ps = plane_words(G), planes = (uint64_t)G.dirs * G.g, copy_words = planes * ps;
+    const uint64_t narrow = (1ull << 18) + (G.dirs == 2 ? 768 * ps + 256 * planes + copy_words / 8
+                                                        : 4096 * ps + 512 * planes + copy_words * 4);
     const uint64_t most = std::min(std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3), narrow);
     return m < round && m * G.dirs * G.r <= most;
 }
