@@ -767,9 +767,12 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
     // (of other directions, of a longer round) lies there by then: from the
     // first captured round on, every round of the handle is counted and its
     // plane copy is always taken to hold bits.
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    SD_CK(rep, cudaStreamIsCapturing(s, &capture));
-    if (capture != cudaStreamCaptureStatusNone) h->plane_replays = true;
+    // (only a caller's stream can be capturing; asking takes 1 us)
+    if (!rep->own_stream) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        SD_CK(rep, cudaStreamIsCapturing(s, &capture));
+        if (capture != cudaStreamCaptureStatusNone) h->plane_replays = true;
+    }
     for (uint64_t off = 0; off < n; off += round) {
         const uint64_t m = std::min(round, n - off);
         if (plane_direct(G, m, round)) {
