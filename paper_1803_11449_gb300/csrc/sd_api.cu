@@ -726,14 +726,22 @@ static int ensure_plane_bins(sd_handle *owner, uint64_t words) {
 // 8), 0.65 (256, 8, 8), 1.3 (1024, 8, 8), 0.6 (64, 6, 10), 1.0 (512, 5, 11),
 // 1.0 (64, 4, 12), 0.85 to 1.1 (256, 4, 12), 1.3 to 1.9 (1024, 4, 12), 2.2
 // (512, 4, 14), 2.2 to 2.7 (256, 5, 14), 3.6 (1024, 5, 14); one direction 0.46
-// (32, 8, 8), 1.1 (256, 8, 8), 1.0 (64, 6, 10), 2.9 (256, 5, 11), 3.2 (256, 4,
-// 12).  `narrow` is a line near or below these.  (32, 8, 8 with 2^17 pairs and two
-// directions: 102 to 139 us direct and 40 binned.)
-static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
+// (32, 8, 8), 1.0 (64, 6, 10), 1.1 (256, 8, 8).  (32, 8, 8 with 2^17 pairs and
+// two directions: 102 to 139 us direct and 40 binned.)  Worst is a round whose
+// pairs all share their destination, an attack: all bits of a direction in one
+// plane, 80 ns per thousand bit-sets and 512 words.  For one direction that
+// decides (256, 4, 12: 600,000 such pairs 214 us direct, 36 binned; other
+// traffic meets at 3 M).  `narrow` is a line near or below all these.
+//
+// In a batch the members' copies push each other out of L2 while binned rounds
+// overlap on the lanes: 64 core sketches of 300,000 pairs each 1.65 ms direct,
+// 1.47 binned; 20,000 pairs and fewer stay direct by far.
+static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round, bool batched) {
     const uint64_t ps = plane_words(G), planes = (uint64_t)G.dirs * G.g, copy_words = planes * ps;
     const uint64_t narrow = (1ull << 18) + (G.dirs == 2 ? 768 * ps + 256 * planes + copy_words / 8
-                                                        : 4096 * ps + 512 * planes + copy_words * 4);
-    const uint64_t most = std::min(std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3), narrow);
+                                                        : 1024 * ps + 512 * planes);
+    uint64_t most = std::min(std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3), narrow);
+    if (batched) most = std::min<uint64_t>(most, 1ull << 21);
     return m < round && m * G.dirs * G.r <= most;
 }
 
@@ -747,7 +755,7 @@ static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round) {
 // any other round is counted exactly, as is every one of a handle whose rounds
 // are in a graph.
 static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir, uint32_t *bins,
-                        uint64_t bin_words, uint64_t round, cudaStream_t s, sd_handle *rep) {
+                        uint64_t bin_words, uint64_t round, cudaStream_t s, sd_handle *rep, bool batched) {
     Geometry G = h->G;
     PlaneArgs P = h->pa;
     P.bins = bins;
@@ -759,7 +767,7 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
         P.nbins = h->G.g;
         P.planes += (uint64_t)dir * h->G.g * P.ps;
     }
-    if (!plane_direct(G, n, round) && plane_bin_words(G, std::min(round, n)) > bin_words)
+    if (!plane_direct(G, n, round, batched) && plane_bin_words(G, std::min(round, n)) > bin_words)
         return rep->fail(SD_ERR_ARG, "plane update: %llu bin words for rounds of %llu pairs",
                          (unsigned long long)bin_words, (unsigned long long)round);
     // Which layout the device holds is known from the rounds queued here.  A
@@ -775,7 +783,7 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
     }
     for (uint64_t off = 0; off < n; off += round) {
         const uint64_t m = std::min(round, n - off);
-        if (plane_direct(G, m, round)) {
+        if (plane_direct(G, m, round, batched)) {
             SD_CK(rep, launch_plane_direct(pairs + 2 * off, m, G, P, h->num_sms, s));
             launched(1);
             continue;
@@ -841,10 +849,10 @@ static int update_device(sd_handle *h, const uint32_t *pairs, uint64_t n, int di
         int rc = ensure_plane_state(h);
         if (rc != SD_OK) return rc;
         const uint64_t round = 1ull << h->T.plane_round_log2;
-        if (!plane_direct(G, n, round))
+        if (!plane_direct(G, n, round, false))
             rc = ensure_plane_bins(h, plane_bin_words(h->G, round));
         if (rc != SD_OK) return rc;
-        return plane_rounds(h, pairs, n, dir, h->plane_bins, h->plane_bins_words, round, h->stream, h);
+        return plane_rounds(h, pairs, n, dir, h->plane_bins, h->plane_bins_words, round, h->stream, h, false);
     }
     const int frc = freshen_grid(h);
     if (frc != SD_OK) return frc;
@@ -1109,7 +1117,7 @@ static int update_many_planes(sd_handle *const *hs, const uint32_t *const *pairs
         cudaStream_t st = l ? d->lane_stream[l - 1] : d->stream;
         uint32_t *bins = l ? d->lane_bins[l - 1] : d->plane_bins;
         const uint64_t bw = l ? d->lane_bins_words[l - 1] : d->plane_bins_words;
-        rc = plane_rounds(hs[q], pairs[q], ns[q], -1, bins, bw, round, st, d);
+        rc = plane_rounds(hs[q], pairs[q], ns[q], -1, bins, bw, round, st, d, order.size() > 1);
         if (rc != SD_OK) return rc;
     }
     for (uint32_t l = 1; l < lanes; l++) {
