@@ -457,34 +457,29 @@ k_plane_apply(Geometry G, PlaneArgs P, uint32_t nbuf, uint32_t per_block) {
     __shared__ bool s_last;
     const uint32_t NB = P.nbins;
     const uint32_t rw = (1u << G.k) >> 5;
-    // a block takes per_block units (the grid holds enough blocks for every
-    // unit), so that blocks retire as the round proceeds and other streams'
-    // work (a window close) gets SMs in between.  The units are dealt to the
-    // blocks in turn, so that a busy plane's go to different ones.  Their
-    // planes are found at once: a thread's planes lie next to each other, two
-    // loads tell whether one of the block's units is among theirs, and only
-    // then they are gone through.  (2^26 pairs of the core sketch 270 us, 280
-    // with a search for each unit and a shared unit counter; 2^23 pairs of
-    // 4096 512-word planes, update alone, 175 us, 179 with the search and
-    // counter, 190 with consecutive units and every plane's range read by
-    // every block.)
-    const uint32_t x0 = blockIdx.x, step = gridDim.x;
+    // a block takes per_block consecutive units (the grid holds enough
+    // blocks for every unit), so that blocks retire as the round
+    // proceeds and other streams' work (a window close) gets SMs in between.
+    // Their planes are found at once: every thread looks at its planes'
+    // ranges of units, one L2 round trip instead of a search of ten for each
+    // unit (2^26 pairs of the core sketch: 270 us, 280 with searches and a
+    // shared unit counter; 128 KiB planes, one block per SM: 345 and 362).
+    const uint32_t x0 = blockIdx.x * per_block;
     wait_for_previous();
     const uint32_t total = P.unit_start[NB];
-    const uint32_t per = (NB + THREADS - 1) / THREADS;
-    const uint32_t b0 = min(threadIdx.x * per, NB), b1 = min(b0 + per, NB);
-    const uint32_t first = P.unit_start[b0], stop = P.unit_start[b1];
-#pragma unroll
-    for (uint32_t j = 0; j < kApplyUnitsPerBlock; j++) {
-        const uint32_t x = x0 + j * step;
-        if (j >= per_block || x < first || x >= stop) continue;
-        uint32_t b = b0, u0 = first;
-        for (uint32_t u1; (u1 = P.unit_start[b + 1]) <= x; u0 = u1) b++;  // (ends: x < stop)
+    for (uint32_t b = threadIdx.x; b < NB; b += THREADS) {
+        const uint32_t u0 = P.unit_start[b], u1 = P.unit_start[b + 1];
+        if (u1 <= x0 || u0 >= x0 + per_block) continue;
         const uint32_t off = bin_off(P, b), n = min(P.cnt[b], bin_room(P, b));
-        const uint32_t at = (x - u0) * P.unit;
-        s_unit[j] = make_uint4(b, off + at, n - at < P.unit ? n - at : P.unit, 0u);
+#pragma unroll
+        for (uint32_t j = 0; j < kApplyUnitsPerBlock; j++) {
+            const uint32_t x = x0 + j;
+            if (j >= per_block || x < u0 || x >= u1) continue;
+            const uint32_t at = (x - u0) * P.unit;
+            s_unit[j] = make_uint4(b, off + at, n - at < P.unit ? n - at : P.unit, 0u);
+        }
     }
-    for (uint32_t it = 0; it < per_block && x0 + it * step < total; it++) {
+    for (uint32_t it = 0; it < per_block && x0 + it < total; it++) {
         uint4 *pl4 = pl4_all + (size_t)(it % nbuf) * (P.ps / 4);
         uint32_t *pl = reinterpret_cast<uint32_t *>(pl4);
         if (threadIdx.x == 0) {
