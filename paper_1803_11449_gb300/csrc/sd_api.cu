@@ -800,7 +800,7 @@ static int plane_rounds(sd_handle *h, const uint32_t *pairs, uint64_t n, int dir
             P.shift = 0;
             if (usable) L = kLayoutScale;
         }
-        SD_CK(rep, launch_plane_round(pairs + 2 * off, m, G, P, h->num_sms, s, L, prev));
+        SD_CK(rep, launch_plane_round(pairs + 2 * off, m, G, P, h->num_sms, s, L, prev, batched));
         launched(L == kLayoutReuse ? 2 : 3);
         h->plane_prev_pairs = m;
         h->plane_layout_view = dir;

@@ -313,8 +313,9 @@ size_t plane_bin_smem_bytes(uint32_t tile_pairs, uint32_t dirs, uint32_t nbins);
 // power of two: a longer round needs no launch for its layout where the bins
 // have that room.
 enum PlaneLayout { kLayoutReuse = 0, kLayoutScale = 1, kLayoutCount = 2 };
+// `lanes`: other rounds run beside this one on other streams (a batch).
 cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
-                               cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs);
+                               cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs, bool lanes);
 // a short round without bins: the n pairs' bits ORed into the plane copy in place
 cudaError_t launch_plane_direct(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
                                 cudaStream_t s);

@@ -637,7 +637,7 @@ static cudaError_t launch_plane_bin_d(const uint32_t *pairs, uint64_t n, const G
 
 template <int R>
 static cudaError_t launch_plane_apply(const Geometry &G, const PlaneArgs &P, uint64_t n, int num_sms,
-                                     cudaStream_t s) {
+                                     cudaStream_t s, bool lanes) {
     // two plane buffers of 512 threads where they fit; one plane of 1024
     // threads per block beyond that
     const bool two = (size_t)P.ps * 8 <= (size_t)100 * 1024;
@@ -663,8 +663,10 @@ static cudaError_t launch_plane_apply(const Geometry &G, const PlaneArgs &P, uin
     // SM of its own.  Set up beside k_plane_bin's blocks, several land on one
     // (700,001 pairs in two directions, update alone: 64-word planes 96 us as
     // dependents and 46 plain, 192 words 45 and 35; 512 words 34 and 36, 8192
-    // words 42 and 42, 2^21 pairs 54 and 56).
-    if (P.ps < kDependentPlaneWords)
+    // words 42 and 42, 2^21 pairs 54 and 56).  On the lanes of a batch, blocks
+    // that wait for their own lane's binning keep another lane's off the SM
+    // (64 core sketches of 500,000 pairs 1.59 ms as dependents, 1.51 plain).
+    if (lanes || P.ps < kDependentPlaneWords)
         return cudaLaunchKernel(reinterpret_cast<const void *>(kern), dim3((unsigned)blocks), dim3(threads), args,
                                 plane * nbuf, s);
     return launch_dependent(reinterpret_cast<const void *>(kern), dim3((unsigned)blocks), dim3(threads), plane * nbuf, s,
@@ -672,7 +674,7 @@ static cudaError_t launch_plane_apply(const Geometry &G, const PlaneArgs &P, uin
 }
 
 cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry &G, const PlaneArgs &P, int num_sms,
-                               cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs) {
+                               cudaStream_t s, PlaneLayout layout, uint64_t prev_pairs, bool lanes) {
     if (n == 0) return cudaSuccess;
     // pairs that start 8 bytes past a 16-byte boundary: the first one is set
     // directly, the rest is read in 16-byte loads (4,000,000 of them: bin 35
@@ -701,12 +703,12 @@ cudaError_t launch_plane_round(const uint32_t *pairs, uint64_t n, const Geometry
                                 : launch_plane_bin_d<1>(pairs, n, G, P, head, num_sms, s);
     if (e != cudaSuccess) return e;
     switch (G.r) {
-        case 3: return launch_plane_apply<3>(G, P, n, num_sms, s);
-        case 4: return launch_plane_apply<4>(G, P, n, num_sms, s);
-        case 5: return launch_plane_apply<5>(G, P, n, num_sms, s);
-        case 6: return launch_plane_apply<6>(G, P, n, num_sms, s);
-        case 7: return launch_plane_apply<7>(G, P, n, num_sms, s);
-        case 8: return launch_plane_apply<8>(G, P, n, num_sms, s);
+        case 3: return launch_plane_apply<3>(G, P, n, num_sms, s, lanes);
+        case 4: return launch_plane_apply<4>(G, P, n, num_sms, s, lanes);
+        case 5: return launch_plane_apply<5>(G, P, n, num_sms, s, lanes);
+        case 6: return launch_plane_apply<6>(G, P, n, num_sms, s, lanes);
+        case 7: return launch_plane_apply<7>(G, P, n, num_sms, s, lanes);
+        case 8: return launch_plane_apply<8>(G, P, n, num_sms, s, lanes);
         default: return cudaErrorInvalidValue;
     }
 }
