@@ -726,12 +726,13 @@ static int ensure_plane_bins(sd_handle *owner, uint64_t words) {
 // 8), 0.65 (256, 8, 8), 1.3 (1024, 8, 8), 0.6 (64, 6, 10), 1.0 (512, 5, 11),
 // 1.0 (64, 4, 12), 0.85 to 1.1 (256, 4, 12), 1.3 to 1.9 (1024, 4, 12), 2.2
 // (512, 4, 14), 2.2 to 2.7 (256, 5, 14), 3.6 (1024, 5, 14); one direction 0.46
-// (32, 8, 8), 1.0 (64, 6, 10), 1.1 (256, 8, 8).  (32, 8, 8 with 2^17 pairs and
+// (32, 8, 8), 1.1 (256, 8, 8), 1.0 (64, 6, 10), 2.9 (256, 5, 11), 3.2 (256, 4,
+// 12).  `narrow` is a line near or below these.  (32, 8, 8 with 2^17 pairs and
 // two directions: 102 to 139 us direct and 40 binned.)  Worst is a round whose
-// pairs all share their destination, an attack: all bits of a direction in one
-// plane, 80 ns per thousand bit-sets and 512 words.  For one direction that
-// decides (256, 4, 12: 600,000 such pairs 214 us direct, 36 binned; other
-// traffic meets at 3 M).  `narrow` is a line near or below all these.
+// pairs all share their destination: all bits of a direction in one plane.
+// The line for two directions holds for that too; with one direction 600,000
+// such pairs of (256, 4, 12) take 214 us directly and 36 binned, while a flow of
+// half of the packets takes 19 directly and 87 binned.
 //
 // In a batch the members' copies push each other out of L2 while binned rounds
 // overlap on the lanes: 64 core sketches of 300,000 pairs each 1.65 ms direct,
@@ -739,7 +740,7 @@ static int ensure_plane_bins(sd_handle *owner, uint64_t words) {
 static bool plane_direct(const Geometry &G, uint64_t m, uint64_t round, bool batched) {
     const uint64_t ps = plane_words(G), planes = (uint64_t)G.dirs * G.g, copy_words = planes * ps;
     const uint64_t narrow = (1ull << 18) + (G.dirs == 2 ? 768 * ps + 256 * planes + copy_words / 8
-                                                        : 1024 * ps + 512 * planes);
+                                                        : 4096 * ps + 512 * planes + copy_words * 4);
     uint64_t most = std::min(std::min<uint64_t>(1ull << 23, (3ull << 20) + copy_words / 3), narrow);
     if (batched) most = std::min<uint64_t>(most, 1ull << 21);
     return m < round && m * G.dirs * G.r <= most;
